@@ -1,12 +1,7 @@
 // Axis permutation of a row-major tensor (the "T" of TTGT, Section 5.1): out axis t = in axis
 // perm[t].  Moves bytes only, so it is exact for any payload.  Axes that stay adjacent and in
-// order are fused first.  When the innermost axis survives the permutation, the tensor is a set
-// of contiguous rows moved as wholes: a group of lanes per row, whose first lane computes the
-// row's source offset and broadcasts it with a shuffle, copies the row in 16-byte vectors when both
-// ends are 16-byte aligned (element by element otherwise).  Otherwise a tile of
-// (output-innermost, input-innermost) is staged in shared memory so that both the reads and the
-// writes are coalesced: 64 x 64 for elements of up to 8 bytes (contiguous runs of 512 bytes on
-// both sides for 8-byte elements, instead of 256), 32 x 32 otherwise.
+// order are fused first, and a surviving innermost axis widens the element (up to 16 bytes) where
+// the buffers are aligned for it.  One kernel then moves tiles: see TilePerm.
 #include <algorithm>
 #include <cstdint>
 #include <vector>
@@ -20,308 +15,349 @@ namespace {
 constexpr int kMaxRank = 32;
 
 struct PermPlan {
-    int32_t rank;                 // fused output rank
+    int32_t rank;                 // fused output rank, without the surviving innermost axis
     int64_t odim[kMaxRank];       // output dims, axis 0 slowest
     int64_t istride[kMaxRank];    // input stride of each output axis
     int64_t ostride[kMaxRank];    // output stride of each output axis
-    int32_t a;                    // output-innermost axis (index into the arrays above)
-    int32_t b;                    // axis that is innermost in the input (-1 if same as a)
+    int64_t inner;                // extent of the innermost axis where it survives (stride 1 on both sides), else 1
     int64_t total;
-    int32_t pow2;                 // every output dim is a power of two: digits by shift and mask
-    int32_t lg[kMaxRank];         // log2 of each output dim (pow2 only)
 };
 
-// Input offset of output row r (all axes but the innermost, p.a); the digits come out by shift
-// and mask when every dim is a power of two.
-__device__ __forceinline__ int64_t row_src(const PermPlan &p, int64_t r) {
-    int64_t src = 0;
-    if (p.pow2) {
-        for (int32_t t = p.rank - 1; t >= 0; --t) {
-            if (t == p.a) continue;
-            src += (r & (p.odim[t] - 1)) * p.istride[t];
-            r >>= p.lg[t];
-        }
-    } else {
-        for (int32_t t = p.rank - 1; t >= 0; --t) {
-            if (t == p.a) continue;
-            const int64_t dgt = r % p.odim[t];
-            r /= p.odim[t];
-            src += dgt * p.istride[t];
-        }
+// One tile: `inner` (or a chunk of it) x group A x group B x group C.  A is a run of the output's
+// innermost axes, B a run of the input's innermost axes outside A, C further axes of the output
+// that fill the tile where A and B cannot (they block each other in a swap of two short axes; they
+// are not needed when the surviving inner run is long).  The last axis of each group may be cut into
+// chunks; the chunk numbers and all other axes form the tile index.  A block reads a tile with
+// consecutive threads along (inner, B) -- contiguous in the input -- and writes it along (inner, A)
+// -- contiguous in the output -- through shared memory, or straight from registers when the two
+// orders agree (no A or no B).
+// Bound by HBM.  Everything that depends on the position inside the tile (two offsets and a
+// shared-memory index per element) is computed once per block, which then moves up to kTileRun
+// tiles: only a base changes from tile to tile, the next tile's loads are in flight while the
+// current one is written, and tiles of 8 to 16 KB leave room for several blocks per SM.  Measured on
+// 2^26 complex64: all axes reversed 169 us, 6.4 TB/s (297 us with 64 x 64 tiles, one per block, whose
+// indices were divided out per element); reversed but for rows of 16 to 512 bytes 164-176 us (470-860
+// us when each row was copied by a group of lanes); (37, 5, 129, 3, 61) complex128 shuffled 29 us
+// (70 us with 32 x 32 tiles of one axis pair, mostly empty).
+struct TilePerm {
+    int32_t ti, ta, tb, tc;                     // tile edges
+    int32_t pitch;                              // shared-memory row of tb * ti elements, odd
+    int32_t direct;                             // read and write order agree: no shared memory
+    uint32_t mi, ma, mb;                        // ceil(2^32 / edge), 0 for an edge of 1
+    int32_t na, nb, nc, nr;                     // axes of each group, innermost first, and of the tile index
+    int32_t adim[kMaxRank], bdim[kMaxRank], cdim[kMaxRank];   // extents inside the tile
+    int64_t ain[kMaxRank], bout[kMaxRank], cin[kMaxRank], cout[kMaxRank];
+    uint32_t rdim[kMaxRank + 4], rbelow[kMaxRank + 4];        // tile index: dims, product of those before
+    int64_t rin[kMaxRank + 4], rout[kMaxRank + 4];
+    int32_t cut[4];                             // tile-index axis that numbers the chunks of inner, A, B, C (-1: whole)
+    int64_t cutdim[4];                          // the cut axis' extent
+    int32_t cutlen[4];                          // and its chunk length
+    int32_t before[4];                          // product of the group's tile extents before the cut axis
+    uint32_t n_tiles;
+    int32_t run;                                // tiles per block
+};
+constexpr int kTileRun = 8;    // most tiles per block
+constexpr int kTileEdge = 32;  // elements of the runs on both sides
+
+// Quotient of e < 2^16 by an edge d <= 2^12 from m = ceil(2^32 / d): exact, as e d < 2^32.
+__device__ __forceinline__ uint32_t quot(uint32_t e, uint32_t m) { return m ? __umulhi(e, m) : e; }
+
+__device__ __forceinline__ int64_t digits_off(int32_t idx, int32_t n, const int32_t *dim, const int64_t *str) {
+    int64_t off = 0;
+    for (int32_t t = 0; t < n; ++t) {
+        const int32_t q = idx / dim[t];
+        off += (int64_t)(idx - q * dim[t]) * str[t];
+        idx = q;
     }
-    return src;
+    return off;
 }
 
-// Row copy: the output is rows of length odim[a] (the fused innermost axis, stride 1 on both
-// sides).  A group of G lanes (G = 16-byte vectors per row, at most 32, a power of two) moves one
-// row: its first lane computes the row's source offset and shares it with a shuffle, and the group
-// copies the row in 16-byte vectors (element by element when a row is not 16-byte aligned).
-template <typename E>
-__global__ void __launch_bounds__(256) k_perm_rows(const E *__restrict__ in, E *__restrict__ out, PermPlan p,
-                                                   int32_t G) {
-    const int lane = threadIdx.x & 31, sub = lane & (G - 1), grp = lane / G;
-    const int64_t len = p.odim[p.a], rows = p.total / len;
-    const int64_t groups = (int64_t)gridDim.x * (blockDim.x >> 5) * (32 / G);
-    const bool vec = (len * (int64_t)sizeof(E)) % 16 == 0 && sizeof(E) <= 16 &&
-                     (reinterpret_cast<uintptr_t>(in) % 16) == 0 && (reinterpret_cast<uintptr_t>(out) % 16) == 0;
-    constexpr int per = 16 / sizeof(E) > 0 ? 16 / (int)sizeof(E) : 1;   // elements per 16-byte vector
-    const int64_t first = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (32 / G) + grp;
-    // every lane runs the same number of iterations (the shuffle needs the whole warp)
-    const int64_t iters = (rows + groups - 1) / groups;
-    for (int64_t it = 0; it < iters; ++it) {
-        const int64_t r = first + it * groups;
-        int64_t src = 0;
-        if (sub == 0 && r < rows) src = row_src(p, r);
-        src = __shfl_sync(0xffffffffu, src, lane - sub);
-        if (r >= rows) continue;
-        const E *ip = in + src;
-        E *op = out + r * len;
-        if (vec) {
-            const uint4 *iv = reinterpret_cast<const uint4 *>(ip);
-            uint4 *ov = reinterpret_cast<uint4 *>(op);
-            const int64_t nv = len / per;
-            for (int64_t i = sub; i < nv; i += G) ov[i] = __ldg(iv + i);
-        } else {
-            for (int64_t i = sub; i < len; i += G) op[i] = __ldg(ip + i);
-        }
-    }
-}
-
-// Short rows (fewer than 64 bytes): one thread per row, copying it element by element; the
-// threads of a warp write consecutive rows, so the writes stay coalesced.
-template <typename E>
-__global__ void __launch_bounds__(256) k_perm_short_rows(const E *__restrict__ in, E *__restrict__ out,
-                                                         PermPlan p) {
-    const int64_t len = p.odim[p.a], rows = p.total / len;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows;
-         r += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t src = row_src(p, r);
-        for (int64_t i = 0; i < len; ++i) out[r * len + i] = __ldg(in + src + i);
-    }
-}
-
-template <typename E>
+// RAGGED: some cut axis has a short last chunk.  O: type of the offsets inside a tile.
+template <typename E, int PER, bool RAGGED, typename O>
 __global__ void __launch_bounds__(256) k_perm_tile(const E *__restrict__ in, E *__restrict__ out,
-                                                   PermPlan p, int64_t tiles_a, int64_t tiles_b) {
-    __shared__ E tile[32][33];
-    const int64_t da = p.odim[p.a], db = p.odim[p.b];
-    int64_t blk = blockIdx.x;
-    const int64_t ta = blk % tiles_a;
-    blk /= tiles_a;
-    const int64_t tb = blk % tiles_b;
-    int64_t batch = blk / tiles_b;
-    int64_t ibase = 0, obase = 0;
-    for (int32_t t = p.rank - 1; t >= 0; --t) {
-        if (t == p.a || t == p.b) continue;
-        int64_t dgt = batch % p.odim[t];
-        batch /= p.odim[t];
-        ibase += dgt * p.istride[t];
-        obase += dgt * p.ostride[t];
+                                                   const __grid_constant__ TilePerm g) {
+    extern __shared__ __align__(16) char dyn[];
+    __shared__ int64_t s_base[kTileRun][2];
+    __shared__ ushort4 s_lim[kTileRun];   // extents of each tile in inner, A, B, C where short of the edges
+    __shared__ int32_t s_edge[kTileRun];  // some extent is short
+    int64_t *s_a = reinterpret_cast<int64_t *>(dyn);
+    int64_t *s_b = s_a + g.ta, *s_ci = s_b + g.tb, *s_co = s_ci + g.tc;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t t0 = blockIdx.x * (uint32_t)g.run, nt = min((uint32_t)g.run, g.n_tiles - t0);
+    // tile bases: a warp per tile, a lane per axis of the tile index (at most 36: two rounds)
+    for (uint32_t t = warp; t < nt; t += 8) {
+        int64_t si = 0, so = 0;
+        uint32_t short_axes = 0;
+        uint16_t lim[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) lim[q] = 0xffff;
+        for (int x = lane; x < g.nr; x += 32) {
+            const uint32_t d = ((t0 + t) / g.rbelow[x]) % g.rdim[x];
+            si += (int64_t)d * g.rin[x];
+            so += (int64_t)d * g.rout[x];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (g.cut[q] == x) {
+                    const int64_t left = g.cutdim[q] - (int64_t)d * g.cutlen[q];
+                    if (left < g.cutlen[q]) {
+                        lim[q] = (uint16_t)(left * g.before[q]);
+                        short_axes = 1;
+                    }
+                }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            si += __shfl_xor_sync(0xffffffffu, si, o);
+            so += __shfl_xor_sync(0xffffffffu, so, o);
+        }
+        const int edge = __any_sync(0xffffffffu, short_axes != 0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) lim[q] = (uint16_t)__reduce_min_sync(0xffffffffu, (unsigned)lim[q]);
+        if (lane == 0) {
+            s_base[t][0] = si;
+            s_base[t][1] = so;
+            s_lim[t] = make_ushort4(lim[0], lim[1], lim[2], lim[3]);
+            s_edge[t] = edge;
+        }
     }
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8 threads
-    const int64_t a0 = ta * 32, b0 = tb * 32;
-    // read: consecutive threads walk the input-innermost axis b (input stride 1)
-    for (int r = ty; r < 32; r += 8) {
-        int64_t ai = a0 + r, bi = b0 + tx;
-        if (ai < da && bi < db) tile[r][tx] = in[ibase + ai * p.istride[p.a] + bi];
+    // the input offset of each A index, the output offset of each B index, both of each C index
+    for (int i = tid; i < g.ta + g.tb + g.tc; i += 256) {
+        if (i < g.ta) {
+            s_a[i] = digits_off(i, g.na, g.adim, g.ain);
+        } else if (i < g.ta + g.tb) {
+            s_b[i - g.ta] = digits_off(i - g.ta, g.nb, g.bdim, g.bout);
+        } else {
+            s_ci[i - g.ta - g.tb] = digits_off(i - g.ta - g.tb, g.nc, g.cdim, g.cin);
+            s_co[i - g.ta - g.tb] = digits_off(i - g.ta - g.tb, g.nc, g.cdim, g.cout);
+        }
     }
     __syncthreads();
-    // write: consecutive threads walk the output-innermost axis a (output stride 1)
-    for (int r = ty; r < 32; r += 8) {
-        int64_t bi = b0 + r, ai = a0 + tx;
-        if (ai < da && bi < db) out[obase + bi * p.ostride[p.b] + ai] = tile[tx][r];
+    // per element of this thread: where it is read (order c, a, b, i) and written (order c, b, a, i)
+    const uint32_t ti = g.ti, ta = g.ta, tb = g.tb, n = ti * ta * tb * (uint32_t)g.tc;
+    O rd[PER], wr[PER];
+    uint32_t sr[PER];        // shared-memory indices: store at the low half, load from the high half
+    uint2 dr[PER], dw[PER];  // indices in inner, A, B, C, against s_lim
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const uint32_t e = tid + u * 256;
+        rd[u] = wr[u] = -1;
+        sr[u] = 0;
+        if (RAGGED) dr[u] = dw[u] = make_uint2(0, 0);
+        if (e < n) {
+            uint32_t q = quot(e, g.mi), i = e - q * ti, q2 = quot(q, g.mb), b = q - q2 * tb, c = quot(q2, g.ma),
+                     a = q2 - c * ta;
+            rd[u] = (O)(s_a[a] + s_ci[c] + b * ti + i);
+            sr[u] = (c * ta + a) * (uint32_t)g.pitch + b * ti + i;
+            if (RAGGED) dr[u] = make_uint2(i | a << 16, b | c << 16);
+            q2 = quot(q, g.ma), a = q - q2 * ta, c = quot(q2, g.mb), b = q2 - c * tb;
+            wr[u] = (O)(s_b[b] + s_co[c] + a * ti + i);
+            sr[u] |= ((c * ta + a) * (uint32_t)g.pitch + b * ti + i) << 16;
+            if (RAGGED) dw[u] = make_uint2(i | a << 16, b | c << 16);
+        }
+    }
+    __syncthreads();   // the offset tables give way to the tile
+    E *tile = reinterpret_cast<E *>(dyn);
+    // inside the extents of tile t (all of it unless the tile is at an edge)
+    auto inside = [&](uint32_t t, const uint2 &d) {
+        if (!RAGGED || !s_edge[t]) return true;
+        const ushort4 l = s_lim[t];
+        return (d.x & 0xffffu) < l.x && (d.x >> 16) < l.y && (d.y & 0xffffu) < l.z && (d.y >> 16) < l.w;
+    };
+    E v[PER];
+    auto load = [&](uint32_t t) {
+        const E *src = in + s_base[t][0];
+#pragma unroll
+        for (int u = 0; u < PER; ++u)
+            if (rd[u] >= 0 && inside(t, dr[u])) v[u] = __ldg(src + rd[u]);
+    };
+    load(0);
+    for (uint32_t t = 0; t < nt; ++t) {
+        E *dst = out + s_base[t][1];
+        if (g.direct) {
+#pragma unroll
+            for (int u = 0; u < PER; ++u)
+                if (wr[u] >= 0 && inside(t, dw[u])) dst[wr[u]] = v[u];
+            if (t + 1 < nt) load(t + 1);
+            continue;
+        }
+#pragma unroll
+        for (int u = 0; u < PER; ++u)
+            if (rd[u] >= 0) tile[sr[u] & 0xffffu] = v[u];
+        __syncthreads();
+        if (t + 1 < nt) load(t + 1);
+#pragma unroll
+        for (int u = 0; u < PER; ++u)
+            if (wr[u] >= 0 && inside(t, dw[u])) dst[wr[u]] = tile[sr[u] >> 16];
+        if (t + 1 < nt) __syncthreads();
     }
 }
 
-// Grouped tile, for permutations of many short axes (the bit permutations of qubit tensors): the
-// output's innermost axes whose sizes multiply to at most 64 (or 32) form group A, the input's
-// innermost axes (outside A) group B.  A block moves PA x PB tiles of (A index, B index), each for
-// one index of the remaining axes, through shared memory: it reads with consecutive threads along B
-// (contiguous in the input) and writes with consecutive threads along A (contiguous in the output).
-constexpr int kGroupMax = 64;   // largest group: the edge of the large tile
-
-struct GroupTile {
-    int32_t pa, pb;                           // sizes of the two groups (products of their dims)
-    int32_t nrest;
-    int64_t in_a[kGroupMax], out_a[kGroupMax];   // offsets of each A index in the input / output
-    int64_t in_b[kGroupMax], out_b[kGroupMax];   // same for B
-    int64_t rdim[kMaxRank], rin[kMaxRank], rout[kMaxRank];   // remaining axes, outermost first
-};
-
-// TE: tile edge (groups of at most TE elements); kTiles tiles per block, TE * TE / 256 elements of
-// each per thread.
-template <typename E, int TE, int kTiles>
-__global__ void __launch_bounds__(256) k_perm_group_tile(const E *__restrict__ in, E *__restrict__ out,
-                                                         const GroupTile g, int64_t n_tiles) {
-    constexpr int kPer = TE * TE / 256;
-    static_assert(kPer * 256 == TE * TE && TE <= kGroupMax && TE + kTiles <= 256, "tile split");
-    __shared__ E tile[TE][TE + 1];
-    __shared__ int64_t s_in_a[TE], s_out_a[TE], s_in_b[TE], s_out_b[TE], s_ib[kTiles], s_ob[kTiles];
-    const int tid = threadIdx.x;
-    // the offset tables move from the parameters to shared memory once (the arithmetic loops index
-    // them per thread), and the next kTiles threads decompose the block's tile indices
-    if (tid < TE) {
-        s_in_a[tid] = tid < g.pa ? g.in_a[tid] : 0;
-        s_out_a[tid] = tid < g.pa ? g.out_a[tid] : 0;
-        s_in_b[tid] = tid < g.pb ? g.in_b[tid] : 0;
-        s_out_b[tid] = tid < g.pb ? g.out_b[tid] : 0;
-    } else if (tid < TE + kTiles) {
-        int64_t blk = (int64_t)blockIdx.x * kTiles + (tid - TE), ib = 0, ob = 0;
-        for (int32_t t = g.nrest - 1; t >= 0; --t) {
-            const int64_t dgt = blk % g.rdim[t];
-            blk /= g.rdim[t];
-            ib += dgt * g.rin[t];
-            ob += dgt * g.rout[t];
-        }
-        s_ib[tid - TE] = ib;
-        s_ob[tid - TE] = ob;
-    }
-    __syncthreads();
-    // every read of the block's tiles is issued first (kTiles x kPer loads in flight per thread),
-    // then each tile goes through shared memory in turn
-    const int n = g.pa * g.pb;                       // at most TE * TE: kPer per thread
-    int nq = kTiles;
-    if ((int64_t)blockIdx.x * kTiles + nq > n_tiles) nq = (int)(n_tiles - (int64_t)blockIdx.x * kTiles);
-    E v[kTiles][kPer];
-#pragma unroll
-    for (int q = 0; q < kTiles; ++q)
-#pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-            const int e = tid + u * 256;
-            if (q < nq && e < n) {
-                const int b = e % g.pb, a = e / g.pb;
-                v[q][u] = __ldg(in + s_ib[q] + s_in_a[a] + s_in_b[b]);
-            }
-        }
-#pragma unroll
-    for (int q = 0; q < kTiles; ++q) {
-        if (q >= nq) break;   // block-uniform
-#pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-            const int e = tid + u * 256;
-            if (e < n) tile[e / g.pb][e % g.pb] = v[q][u];
-        }
-        __syncthreads();
-        const int64_t ob = s_ob[q];
-        for (int e = tid; e < n; e += blockDim.x) {
-            const int a = e % g.pa, b = e / g.pa;
-            out[ob + s_out_a[a] + s_out_b[b]] = tile[a][b];
-        }
-        __syncthreads();
-    }
-}
-
-// Builds the grouped tile of plan p with groups of at most `lim` elements (lim <= kGroupMax); false
-// when it does not apply (groups smaller than 8 elements).
-bool group_tile(const PermPlan &p, GroupTile &g, int64_t lim) {
-    std::vector<char> in_a(p.rank, 0), in_b(p.rank, 0);
-    int64_t pa = 1, pb = 1;
-    std::vector<int32_t> ga, gb;   // innermost first
-    for (int32_t t = p.rank - 1; t >= 0 && pa * p.odim[t] <= lim; --t) {
-        pa *= p.odim[t];
-        ga.push_back(t);
-        in_a[t] = 1;
-    }
-    // input order: axes by decreasing input stride; group B takes the innermost ones outside A
-    std::vector<int32_t> by_in(p.rank);
+// Builds the tiles of plan p: runs of about `edge` elements on both sides, at most `area` elements.
+// false if the tensor has too many of them.
+bool tile_perm(const PermPlan &p, int32_t edge, int32_t area, TilePerm &g) {
+    std::vector<char> used(p.rank, 0);
+    std::vector<int32_t> by_in(p.rank);  // axes by increasing input stride
     for (int32_t t = 0; t < p.rank; ++t) by_in[t] = t;
     std::sort(by_in.begin(), by_in.end(), [&](int32_t x, int32_t y) { return p.istride[x] < p.istride[y]; });
-    for (int32_t t : by_in) {
-        if (in_a[t]) continue;
-        if (pb * p.odim[t] > lim) break;
-        pb *= p.odim[t];
-        gb.push_back(t);
-        in_b[t] = 1;
+    struct Axis { int64_t dim, in, out; };
+    std::vector<Axis> A, B, C, R;
+    // an edge of at most t splits n indices into chunks of equal length
+    auto chunk = [](int64_t n, int64_t t) {
+        const int64_t c = (n + t - 1) / t;
+        return (n + c - 1) / c;
+    };
+    auto prod = [](const std::vector<Axis> &v) {
+        int64_t x = 1;
+        for (const Axis &a : v) x *= a.dim;
+        return x;
+    };
+    int32_t ia = p.rank - 1, ib = 0;
+    auto take = [&](std::vector<Axis> &v, int32_t t) {
+        v.push_back({p.odim[t], p.istride[t], p.ostride[t]});
+        used[t] = 1;
+    };
+    auto grow_a = [&](int64_t lim) {
+        if (ia < 0 || used[ia] || prod(A) >= lim) return false;
+        take(A, ia--);
+        return true;
+    };
+    auto grow_b = [&](int64_t lim) {
+        if (ib >= p.rank || used[by_in[ib]] || prod(B) >= lim) return false;
+        take(B, by_in[ib++]);
+        return true;
+    };
+    for (int q = 0; q < 4; ++q) {
+        g.cut[q] = -1;
+        g.cutdim[q] = 0;
+        g.cutlen[q] = 1;
+        g.before[q] = 1;
     }
-    if (pa < 8 || pb < 8) return false;
-    g.pa = (int32_t)pa;
-    g.pb = (int32_t)pb;
-    auto offsets = [&](const std::vector<int32_t> &axes, int64_t *oin, int64_t *oout, int64_t n) {
-        for (int64_t idx = 0; idx < n; ++idx) {
-            int64_t rem = idx, si = 0, so = 0;
-            for (int32_t t : axes) {   // innermost first
-                const int64_t d = rem % p.odim[t];
-                rem /= p.odim[t];
-                si += d * p.istride[t];
-                so += d * p.ostride[t];
-            }
-            oin[idx] = si;
-            oout[idx] = so;
+    // cuts the last axis of a group so that its extent is at most lim
+    auto cut = [&](std::vector<Axis> &v, int64_t lim, int q) {
+        if (v.empty()) return;
+        Axis &last = v.back();
+        const int64_t before = prod(v) / last.dim, len = chunk(last.dim, std::max<int64_t>(1, lim / before));
+        if (len < last.dim) {
+            R.push_back({(last.dim + len - 1) / len, last.in * len, last.out * len});
+            g.cutdim[q] = last.dim;
+            g.cutlen[q] = (int32_t)len;
+            g.cut[q] = (int32_t)R.size() - 1;   // index into R, renumbered below
+            g.before[q] = (int32_t)before;
+            last.dim = len;
         }
     };
-    offsets(ga, g.in_a, g.out_a, pa);
-    offsets(gb, g.in_b, g.out_b, pb);
-    g.nrest = 0;
-    for (int32_t t = 0; t < p.rank; ++t) {
-        if (in_a[t] || in_b[t]) continue;
-        g.rdim[g.nrest] = p.odim[t];
-        g.rin[g.nrest] = p.istride[t];
-        g.rout[g.nrest] = p.ostride[t];
-        g.nrest++;
+    int64_t ti = p.inner;
+    if (ti > area) {
+        ti = chunk(p.inner, area);
+        R.push_back({(p.inner + ti - 1) / ti, ti, ti});
+        g.cutdim[0] = p.inner;
+        g.cutlen[0] = (int32_t)ti;
+        g.cut[0] = 0;
     }
+    int64_t lim_a = std::max<int64_t>(1, edge / ti), lim_b = std::max<int64_t>(1, area / (ti * lim_a));
+    if (ti >= edge) lim_b = 1;   // long surviving runs: whole rows, in the order of the output (C)
+    for (bool more = true; more;) {   // in turn, so that neither takes all the short axes
+        const bool ga = grow_a(lim_a), gb = grow_b(lim_b);
+        more = ga || gb;
+    }
+    // a group that is blocked short of its edge leaves more of the tile to the other
+    if (ti < edge && prod(A) < lim_a) {
+        lim_b = std::max(lim_b, area / (ti * prod(A)));
+        while (grow_b(lim_b)) {}
+    }
+    if (ti < edge && prod(B) < lim_b) {
+        lim_a = std::max(lim_a, area / (ti * prod(B)));
+        while (grow_a(lim_a)) {}
+    }
+    cut(A, lim_a, 1);
+    cut(B, lim_b, 2);
+    const int64_t ta = prod(A), tb = prod(B), room = std::max<int64_t>(1, area / (ti * ta * tb));
+    for (int32_t t = p.rank - 1; t >= 0 && prod(C) < room; --t)
+        if (!used[t]) take(C, t);
+    cut(C, room, 3);
+    const int64_t tc = prod(C);
+    if (ti * ta * tb * tc > area) return false;
+    g.ti = (int32_t)ti;
+    g.ta = (int32_t)ta;
+    g.tb = (int32_t)tb;
+    g.tc = (int32_t)tc;
+    g.pitch = (int32_t)((tb * ti) | 1);
+    g.direct = ta == 1 || tb == 1;
+    auto magic = [](int64_t d) { return d == 1 ? 0u : (uint32_t)(((uint64_t(1) << 32) + d - 1) / d); };
+    g.mi = magic(ti);
+    g.ma = magic(ta);
+    g.mb = magic(tb);
+    g.na = (int32_t)A.size();
+    g.nb = (int32_t)B.size();
+    g.nc = (int32_t)C.size();
+    for (int32_t i = 0; i < g.na; ++i) { g.adim[i] = (int32_t)A[i].dim; g.ain[i] = A[i].in; }
+    for (int32_t i = 0; i < g.nb; ++i) { g.bdim[i] = (int32_t)B[i].dim; g.bout[i] = B[i].out; }
+    for (int32_t i = 0; i < g.nc; ++i) { g.cdim[i] = (int32_t)C[i].dim; g.cin[i] = C[i].in; g.cout[i] = C[i].out; }
+    // the tile index: chunk numbers and the other axes, innermost in the output first, so that
+    // consecutive tiles write neighbouring runs
+    for (int32_t t = 0; t < p.rank; ++t)
+        if (!used[t]) R.push_back({p.odim[t], p.istride[t], p.ostride[t]});
+    std::vector<int32_t> ord(R.size());
+    for (size_t i = 0; i < ord.size(); ++i) ord[i] = (int32_t)i;
+    std::sort(ord.begin(), ord.end(), [&](int32_t x, int32_t y) { return R[x].out < R[y].out; });
+    g.nr = (int32_t)R.size();
+    int64_t tiles = 1;
+    int32_t cuts[4] = {-1, -1, -1, -1};
+    for (int32_t i = 0; i < g.nr; ++i) {
+        const Axis &x = R[ord[i]];
+        g.rbelow[i] = (uint32_t)tiles;
+        if (x.dim > 0x7fffffffLL || tiles > 0x7fffffffLL / x.dim) return false;
+        tiles *= x.dim;
+        g.rdim[i] = (uint32_t)x.dim;
+        g.rin[i] = x.in;
+        g.rout[i] = x.out;
+        for (int q = 0; q < 4; ++q)
+            if (g.cut[q] == ord[i]) cuts[q] = i;
+    }
+    for (int q = 0; q < 4; ++q) g.cut[q] = cuts[q];
+    g.n_tiles = (uint32_t)tiles;
+    // several tiles per block once every SM has six blocks
+    g.run = (int32_t)std::min<int64_t>(kTileRun, (tiles + 152 * 6 - 1) / (152 * 6));
     return true;
 }
 
-template <typename E>
-cudaError_t perm_launch(const void *src, void *dst, const PermPlan &p, cudaStream_t st) {
-    const E *in = static_cast<const E *>(src);
-    E *out = static_cast<E *>(dst);
-    if (p.total == 0) return cudaSuccess;
-    if (p.b >= 0 && p.odim[p.a] < 32) {
-        GroupTile g;
-        // the 64 x 64 tile (33 KB of shared memory for 8-byte elements) when it is at least half
-        // full, else the 32 x 32 tile, four per block
-        if constexpr (sizeof(E) <= 8) {
-            if (group_tile(p, g, 64) && (int64_t)g.pa * g.pb >= 2048) {
-                const int64_t tiles = p.total / ((int64_t)g.pa * g.pb);
-                if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-                k_perm_group_tile<E, 64, 1><<<(unsigned)tiles, 256, 0, st>>>(in, out, g, tiles);
-                return cudaGetLastError();
-            }
-        }
-        if (group_tile(p, g, 32)) {
-            const int64_t tiles = p.total / ((int64_t)g.pa * g.pb), blocks = (tiles + 3) / 4;
-            if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-            k_perm_group_tile<E, 32, 4><<<(unsigned)blocks, 256, 0, st>>>(in, out, g, tiles);
-            return cudaGetLastError();
-        }
-    }
-    if (p.b < 0) {
-        const int64_t rows = p.total / p.odim[p.a];
-        if (p.odim[p.a] * (int64_t)sizeof(E) < 64) {
-            int64_t blocks = (rows + 255) / 256;
-            if (blocks > 152 * 16) blocks = 152 * 16;
-            k_perm_short_rows<E><<<(unsigned)blocks, 256, 0, st>>>(in, out, p);
-        } else {
-            // G lanes per row (its 16-byte vectors, rounded up to a power of two, at most 32)
-            const int64_t nvec = (p.odim[p.a] * (int64_t)sizeof(E) + 15) / 16;
-            int32_t G = 1;
-            while (G < 32 && G < nvec) G *= 2;
-            const int64_t per_block = 8 * (32 / G);
-            int64_t blocks = (rows + per_block - 1) / per_block;
-            if (blocks > 152 * 8) blocks = 152 * 8;
-            k_perm_rows<E><<<(unsigned)blocks, 256, 0, st>>>(in, out, p, G);
-        }
-    } else {
-        int64_t da = p.odim[p.a], db = p.odim[p.b];
-        int64_t ta = (da + 31) / 32, tb = (db + 31) / 32;
-        int64_t batch = p.total / (da * db);
-        int64_t blocks = ta * tb * batch;
-        if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-        k_perm_tile<E><<<(unsigned)blocks, 256, 0, st>>>(in, out, p, ta, tb);
-    }
+template <typename E, int PER, bool RAGGED, typename O>
+cudaError_t launch_tiles(const E *in, E *out, const TilePerm &g, cudaStream_t st) {
+    const size_t tables = (size_t)(g.ta + g.tb + 2 * g.tc) * 8;
+    const size_t smem = std::max(tables, g.direct ? 0 : (size_t)g.tc * g.ta * g.pitch * sizeof(E));
+    const unsigned blocks = (g.n_tiles + g.run - 1) / g.run;
+    k_perm_tile<E, PER, RAGGED, O><<<blocks, 256, smem, st>>>(in, out, g);
     return cudaGetLastError();
 }
 
-}  // namespace
+// Tiles of 2048 elements of up to 8 bytes where no chunk is short, of 1024 otherwise: a 16-byte element
+// fills 16 KB with 1024, and the bookkeeping of ragged tiles costs registers per element.
+template <typename E>
+cudaError_t perm_launch(const void *src, void *dst, const PermPlan &p, cudaStream_t st) {
+    if (p.total == 0) return cudaSuccess;
+    const E *in = static_cast<const E *>(src);
+    E *out = static_cast<E *>(dst);
+    constexpr int AREA = sizeof(E) <= 8 ? 2048 : 1024;
+    TilePerm g;
+    if (p.total <= 0x7fffffffLL) {
+        if (!tile_perm(p, kTileEdge, AREA, g)) return cudaErrorInvalidValue;
+        bool ragged = false;
+        for (int q = 0; q < 4; ++q) ragged = ragged || (g.cut[q] >= 0 && g.cutdim[q] % g.cutlen[q] != 0);
+        if (!ragged) return launch_tiles<E, AREA / 256, false, int32_t>(in, out, g, st);
+    }
+    if (!tile_perm(p, kTileEdge, 1024, g)) return cudaErrorInvalidValue;
+    if (p.total <= 0x7fffffffLL) return launch_tiles<E, 4, true, int32_t>(in, out, g, st);
+    return launch_tiles<E, 4, true, int64_t>(in, out, g, st);
+}
 
-cudaError_t launch_permute(const void *src, void *dst, int32_t elem_bytes, int32_t rank,
-                           const int64_t *dims, const int32_t *perm, cudaStream_t stream) {
+// The fused plan of a permutation; false if it has too many axes.
+bool perm_plan(int32_t rank, const int64_t *dims, const int32_t *perm, PermPlan &p) {
     // input strides
     std::vector<int64_t> istr(rank);
     int64_t acc = 1;
     for (int32_t t = rank - 1; t >= 0; --t) { istr[t] = acc; acc *= dims[t]; }
-    const int64_t total = acc;
+    p = PermPlan{};
+    p.total = acc;
+    p.inner = 1;
     // output axes (dims of 1 dropped), fused when adjacent in the input in the same order
     std::vector<int64_t> od, is;
     for (int32_t t = 0; t < rank; ++t) {
@@ -335,30 +371,43 @@ cudaError_t launch_permute(const void *src, void *dst, int32_t elem_bytes, int32
             is.push_back(s);
         }
     }
-    PermPlan p{};
-    p.total = total;
+    if (!od.empty() && is.back() == 1) {
+        p.inner = od.back();
+        od.pop_back();
+        is.pop_back();
+    }
     p.rank = (int32_t)od.size();
-    if (p.rank > kMaxRank) return cudaErrorInvalidValue;
-    acc = 1;
+    if (p.rank > kMaxRank) return false;
+    acc = p.inner;
     for (int32_t t = p.rank - 1; t >= 0; --t) {
         p.odim[t] = od[t];
         p.istride[t] = is[t];
         p.ostride[t] = acc;
         acc *= od[t];
     }
-    p.a = p.rank - 1;
-    p.b = -1;
-    if (p.rank >= 2 && p.istride[p.a] != 1) {
-        for (int32_t t = 0; t < p.rank; ++t)
-            if (p.istride[t] == 1) p.b = t;
-    }
-    if (p.rank == 0) { p.rank = 1; p.odim[0] = 1; p.istride[0] = 1; p.ostride[0] = 1; p.a = 0; }
-    p.pow2 = 1;
+    return true;
+}
+
+// Moves elements of `by` times the size where the surviving run is a multiple of it.
+void widen(PermPlan &p, int64_t by) {
+    p.inner /= by;
+    p.total /= by;
     for (int32_t t = 0; t < p.rank; ++t) {
-        int32_t l = 0;
-        while ((int64_t(1) << l) < p.odim[t]) ++l;
-        p.lg[t] = l;
-        if ((int64_t(1) << l) != p.odim[t]) p.pow2 = 0;
+        p.istride[t] /= by;   // multiples of the whole surviving run
+        p.ostride[t] /= by;
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_permute(const void *src, void *dst, int32_t elem_bytes, int32_t rank,
+                           const int64_t *dims, const int32_t *perm, cudaStream_t stream) {
+    PermPlan p;
+    if (!perm_plan(rank, dims, perm, p)) return cudaErrorInvalidValue;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst);
+    while (elem_bytes < 16 && p.inner % 2 == 0 && at % (2 * (uintptr_t)elem_bytes) == 0 && p.total > 0) {
+        widen(p, 2);
+        elem_bytes *= 2;
     }
     switch (elem_bytes) {
         case 1: return perm_launch<uint8_t>(src, dst, p, stream);

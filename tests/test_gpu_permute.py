@@ -57,3 +57,32 @@ def test_permute_rejects_bad_perm(env):
     x = torch.zeros(8, dtype=torch.int64, device="cuda")
     with pytest.raises(tnsa.TnError):
         tnsa.tn_permute(ctx, x.data_ptr(), x.data_ptr(), 8, (2, 4), (0, 0))
+
+
+# edges of the tiles: chunks cut short in every group, groups that block each other, a surviving run
+# that widens the element, one longer than a tile, buffers too badly aligned to widen, more tiles than one
+# block takes
+EDGE_CASES = [
+    ((31, 33, 2), (2, 1, 0), 0), ((129, 3, 61, 5), (3, 1, 0, 2), 0), ((700, 2, 2), (0, 2, 1), 0),
+    ((900, 3, 5), (0, 2, 1), 0), ((3, 4097), (1, 0), 0), ((4097, 3), (1, 0), 0), ((5, 3, 2), (1, 0, 2), 0),
+    ((5, 3, 6), (1, 0, 2), 1), ((3, 2, 5003), (1, 0, 2), 0), ((2,) * 18, tuple(range(17, -1, -1)), 1),
+    ((2,) * 21, tuple(range(14, -1, -1)) + (15, 16, 17, 18, 19, 20), 0), ((300, 300, 40), (2, 1, 0), 0), ((1, 1), (1, 0), 0),
+]
+
+
+@pytest.mark.parametrize("case", range(len(EDGE_CASES)))
+@pytest.mark.parametrize("elem", [1, 2, 4, 8, 16])
+def test_permute_tile_edges(env, case, elem):
+    torch, tnsa, ctx = env
+    dims, perm, shift = EDGE_CASES[case]   # shift: elements by which the buffers miss their alignment
+    n = int(np.prod(dims))
+    src = np.random.default_rng(case).integers(0, 256, (n + shift) * elem, dtype=np.uint8)
+    want = src[shift * elem:].reshape(*dims, elem).transpose(*perm, len(dims)).reshape(-1)
+    d_in = torch.from_numpy(src).cuda()
+    d_out = torch.zeros((n + 2 * shift) * elem, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    tnsa.tn_permute(ctx, d_in.data_ptr() + shift * elem, d_out.data_ptr() + shift * elem, elem, dims, perm)
+    tnsa.tn_ctx_synchronize(ctx)
+    got = d_out.cpu().numpy()
+    assert np.array_equal(got[shift * elem:(n + shift) * elem], want)
+    assert not got[:shift * elem].any() and not got[(n + shift) * elem:].any()
