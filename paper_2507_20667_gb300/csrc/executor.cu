@@ -315,11 +315,19 @@ bool make_lgroups(const std::vector<int64_t> &dim, const std::vector<int64_t> &s
     return true;
 }
 
-// Tabulate the index maps of a small step with at most kTabOut outputs and kTabK shared indices
-// (LFLAG_TAB): the warp then reads each offset instead of decoding the index over the leg groups.
-// The decode is the one the kernels perform (digits by shift and mask, or by division).
+// Prepares a small step: how many lanes share an output (a power of two that splits a long shared
+// index while outputs alone would leave lanes idle), and the tables of its index maps (LFLAG_TAB) --
+// the warp then reads each offset instead of decoding the index over the leg groups.  Tabulated are
+// steps of at most kTabOut outputs and kTabK shared indices, and larger ones whose dims are powers of
+// two (the offset is then a sum over index bits) while the words fit the group fields.  The decode is
+// the one the kernels perform (digits by shift and mask, or by division).
 void tabulate_small(LocalStep &ls) {
-    if (!(ls.flags & LFLAG_SMALL) || (int64_t)ls.M * ls.N > kTabOut || ls.K > kTabK) return;
+    const int64_t O = (int64_t)ls.M * ls.N;
+    if (!(ls.flags & LFLAG_SMALL)) return;
+    while ((2 << ls.lg_split) * O <= 32 && (1 << ls.lg_split) < ls.K) ++ls.lg_split;
+    const int64_t high = O > kTabOut ? (O + kTabOut - 1) / kTabOut : 0;   // words for outputs 16 i
+    if (ls.K > kTabK || kTabOut + ls.K + high > kTabWords || (high && !(ls.pow2 && is_pow2(ls.M) && is_pow2(ls.N))))
+        return;
     auto dec = [&](int32_t n, const int32_t *dim, const int32_t *str, const uint8_t *lsb, int32_t idx) {
         int64_t off = 0;
         for (int32_t i = 0; i < n; ++i) {
@@ -334,19 +342,22 @@ void tabulate_small(LocalStep &ls) {
         }
         return off;
     };
-    uint32_t t[kTabOut + kTabK] = {};
-    for (int32_t o = 0; o < ls.M * ls.N; ++o) {
-        const int64_t a = dec(ls.nm, ls.m_dim, ls.m_str, ls.m_lsb, o / ls.N);
-        const int64_t b = dec(ls.nn, ls.n_dim, ls.n_str, ls.n_lsb, o % ls.N);
-        if (a > 0xffff || b > 0xffff) return;
-        t[o] = (uint32_t)a | ((uint32_t)b << 16);
-    }
-    for (int32_t k = 0; k < ls.K; ++k) {
-        const int64_t a = dec(ls.nk, ls.k_dim, ls.k_sa, ls.k_lsb, k);
-        const int64_t b = dec(ls.nk, ls.k_dim, ls.k_sb, ls.k_lsb, k);
-        if (a > 0xffff || b > 0xffff) return;
-        t[kTabOut + k] = (uint32_t)a | ((uint32_t)b << 16);
-    }
+    uint32_t t[kTabWords] = {};
+    auto put = [&](int32_t w, int64_t a, int64_t b) {
+        t[w] = (uint32_t)a | ((uint32_t)b << 16);
+        return a <= 0xffff && b <= 0xffff;
+    };
+    auto out = [&](int32_t w, int32_t o) {
+        return put(w, dec(ls.nm, ls.m_dim, ls.m_str, ls.m_lsb, o / ls.N),
+                   dec(ls.nn, ls.n_dim, ls.n_str, ls.n_lsb, o % ls.N));
+    };
+    for (int32_t o = 0; o < std::min<int64_t>(O, kTabOut); ++o)
+        if (!out(o, o)) return;
+    for (int32_t k = 0; k < ls.K; ++k)
+        if (!put(kTabOut + k, dec(ls.nk, ls.k_dim, ls.k_sa, ls.k_lsb, k), dec(ls.nk, ls.k_dim, ls.k_sb, ls.k_lsb, k)))
+            return;
+    for (int32_t i = 0; i < high; ++i)
+        if (!out(kTabOut + ls.K + i, i * kTabOut)) return;
     std::memcpy(reinterpret_cast<char *>(&ls) + offsetof(LocalStep, m_dim), t, sizeof(t));
     ls.flags |= LFLAG_TAB;
 }
@@ -577,7 +588,6 @@ bool warp_fit(int32_t v, int32_t n, const Plan &plan, const std::vector<Geom> &g
 // Staging records of one program input (a leaf, or a warp program's result): pieces of at most
 // kStagePiece elements, so that each thread of the staging loop copies one piece with one burst of
 // loads; the first piece carries the input's scale slot and node.
-constexpr int32_t kStagePiece = 16;
 tn_status push_input(std::vector<LeafRef> &out, int64_t goff, int64_t count, int64_t smem_off, int32_t slot,
                      int32_t node, int32_t src) {
     for (int64_t p = 0; p < std::max<int64_t>(count, 1); p += kStagePiece) {

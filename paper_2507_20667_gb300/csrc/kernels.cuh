@@ -78,13 +78,15 @@ enum LocalMode : uint8_t { LMODE_ROWS = 0, LMODE_GEMM = 1, LMODE_REDUCE = 2 };
 enum LocalFlags : int32_t {
     LFLAG_JOB_ROOT = 1,     // (program, step) produces the job's amplitude
     LFLAG_SMALL = 2,        // (step) small enough for one warp
-    LFLAG_TAB = 4,          // (small step, M N <= 16, K <= 16) the index maps are tabulated: the
-                            // bytes of the group fields from m_dim on hold kTabWords packed
-                            // offsets (low 16 bits in A, high 16 in B), outputs then shared indices
+    LFLAG_TAB = 4,          // (small step, see tabulate_small) the index maps are tabulated: the
+                            // bytes of the group fields from m_dim on hold packed offsets (low 16
+                            // bits in A, high 16 in B): of the outputs 0..15, of the shared indices,
+                            // then of the outputs 0, 16, 32, ... (power-of-two steps of more than 16
+                            // outputs: the offset of output o is that of o mod 16 plus that of the rest)
     LFLAG_C_OUT = 16        // (warp programs) C is the program's result: written to the job's
                             // arena at root_c_off
 };
-constexpr int kTabOut = 16, kTabK = 16;
+constexpr int kTabOut = 16, kTabK = 16, kTabWords = 40;
 
 // A wave of a program: steps [first, first + n_small) run one per warp, then n_big steps use the
 // whole block; the steps of a wave are independent of each other.
@@ -104,10 +106,11 @@ struct LocalStep {
     int32_t n_dim[kLG], n_str[kLG];     // free legs of B (stride in B)
     int32_t k_dim[kLG], k_sa[kLG], k_sb[kLG];
     uint8_t m_lsb[kLG], n_lsb[kLG], k_lsb[kLG];
-    uint8_t pad[2];
+    uint8_t lg_split;                   // small steps: log2 of the lanes that share an output
+    uint8_t pad;
 };
 static_assert(sizeof(LocalStep) == 224, "LocalStep layout");
-static_assert(offsetof(LocalStep, m_lsb) - offsetof(LocalStep, m_dim) >= 4 * (kTabOut + kTabK),
+static_assert(offsetof(LocalStep, m_lsb) - offsetof(LocalStep, m_dim) >= 4 * kTabWords,
               "the tabulated offsets fit the group fields");
 
 struct LocalProg {
@@ -127,10 +130,11 @@ struct LocalProg {
 // the wave that consumes it (large subtrees such as fan-in chains).
 enum ProgKind : int32_t { PROG_BLOCK = 0, PROG_WARP = 1, PROG_BIG = 2 };
 
-// A staging piece of a program input: `count` (at most 16) elements at element offset global_off
+// A staging piece of a program input: `count` (at most kStagePiece) elements at element offset global_off
 // of the job's leaf buffer (src 0) or of its arena (src 1: a warp program's result), copied to
 // shared-memory element offset smem_off.  The first piece of an input has slot >= 0 and also
 // copies the max-abs and exponent of node `node` into that scale slot.
+constexpr int32_t kStagePiece = 16;
 struct LeafRef {
     int64_t global_off;
     int32_t count, smem_off, slot, node, src, pad;

@@ -13,64 +13,53 @@
 
 namespace tn {
 
+// Digits by division, out of line (see group_off_div).
+static __device__ __noinline__ int32_t lgroup_off_div(int32_t n, const int32_t *dim, const int32_t *str, int32_t idx) {
+    int32_t off = 0;
+#pragma unroll 1
+    for (int32_t i = 0; i < n; ++i) {
+        const int32_t q = idx / dim[i];
+        off += (idx - q * dim[i]) * str[i];
+        idx = q;
+    }
+    return off;
+}
+static __device__ __noinline__ int2 lgroup_off2_div(const LocalStep *s, int32_t idx) {
+    int2 off = make_int2(0, 0);
+#pragma unroll 1
+    for (int32_t i = 0; i < s->nk; ++i) {
+        const int32_t q = idx / s->k_dim[i], d = idx - q * s->k_dim[i];
+        off.x += d * s->k_sa[i];
+        off.y += d * s->k_sb[i];
+        idx = q;
+    }
+    return off;
+}
+
 __device__ __forceinline__ int32_t lgroup_off(int32_t n, const int32_t *dim, const int32_t *str,
                                               const uint8_t *lsb, bool pow2, int32_t idx) {
+    if (!pow2) return lgroup_off_div(n, dim, str, idx);
     int32_t off = 0;
-    if (pow2) {
-        for (int32_t i = 0; i < n; ++i) off += ((idx >> lsb[i]) & (dim[i] - 1)) * str[i];
-    } else {
-        for (int32_t i = 0; i < n; ++i) {
-            const int32_t d = idx % dim[i];
-            idx /= dim[i];
-            off += d * str[i];
-        }
-    }
+#pragma unroll 1
+    for (int32_t i = 0; i < n; ++i) off += ((idx >> lsb[i]) & (dim[i] - 1)) * str[i];
     return off;
 }
 
 __device__ __forceinline__ void lgroup_off2(const LocalStep &s, int32_t idx, int32_t &oa, int32_t &ob) {
+    if (!s.pow2) {
+        const int2 o = lgroup_off2_div(&s, idx);
+        oa = o.x;
+        ob = o.y;
+        return;
+    }
     oa = 0;
     ob = 0;
-    if (s.pow2) {
-        for (int32_t i = 0; i < s.nk; ++i) {
-            const int32_t d = (idx >> s.k_lsb[i]) & (s.k_dim[i] - 1);
-            oa += d * s.k_sa[i];
-            ob += d * s.k_sb[i];
-        }
-    } else {
-        for (int32_t i = 0; i < s.nk; ++i) {
-            const int32_t d = idx % s.k_dim[i];
-            idx /= s.k_dim[i];
-            oa += d * s.k_sa[i];
-            ob += d * s.k_sb[i];
-        }
+#pragma unroll 1
+    for (int32_t i = 0; i < s.nk; ++i) {
+        const int32_t d = (idx >> s.k_lsb[i]) & (s.k_dim[i] - 1);
+        oa += d * s.k_sa[i];
+        ob += d * s.k_sb[i];
     }
-}
-
-// A power-of-two group list held in registers: offset(idx) = sum ((idx >> lsb) & mask) * stride.
-struct RegGroups {
-    int32_t n;
-    int32_t lsb[kLG], mask[kLG], str[kLG];
-};
-
-__device__ __forceinline__ RegGroups reg_groups(int32_t n, const int32_t *dim, const int32_t *str,
-                                                const uint8_t *lsb) {
-    RegGroups g;
-    g.n = n;
-#pragma unroll
-    for (int i = 0; i < kLG; ++i) {
-        g.lsb[i] = i < n ? lsb[i] : 0;
-        g.mask[i] = i < n ? dim[i] - 1 : 0;
-        g.str[i] = i < n ? str[i] : 0;
-    }
-    return g;
-}
-
-__device__ __forceinline__ int32_t reg_off(const RegGroups &g, int32_t idx) {
-    int32_t off = 0;
-#pragma unroll
-    for (int i = 0; i < kLG; ++i) off += ((idx >> g.lsb[i]) & g.mask[i]) * g.str[i];
-    return off;
 }
 
 constexpr int kKTab = 1024;   // shared indices whose offsets are tabulated per step
@@ -99,29 +88,48 @@ __device__ __forceinline__ LocalSmem local_layout(char *dyn, const LocalProg &P)
     return L;
 }
 
+struct SplitSlots {       // block programs: two arrays
+    uint32_t *smax;
+    int32_t *sexp;
+    __device__ __forceinline__ void put(int32_t i, uint32_t m, int32_t e) const {
+        smax[i] = m;
+        sexp[i] = e;
+    }
+};
+struct PairSlots {        // warp programs: pairs
+    int2 *slot;
+    __device__ __forceinline__ void put(int32_t i, uint32_t m, int32_t e) const {
+        slot[i] = make_int2((int32_t)m, e);
+    }
+};
 // Copies a program's inputs into shared memory: one staging piece (at most 16 elements of a leaf
-// or of a program's result) per thread, its elements loaded in bursts of LB independent loads;
-// the first piece of each input also copies the input's max-abs and exponent.
-template <typename T, int LB = 16>
+// or of a program's result) per thread, its elements loaded in one burst; the first piece of each
+// input also copies the input's max-abs and exponent.  Every thread runs the same number of
+// iterations: lanes that leave the loop at different times need not reconverge, and a warp program
+// then issues all its steps once per group of lanes (measured: steps of programs with more than 32
+// pieces 2.3 times slower).
+template <typename T, typename S>
 __device__ __forceinline__ void stage_inputs(const JobPtrs &j, const LeafRef *refs, int32_t n_refs, int32_t t0,
-                                             int32_t stride, cx_t<T> *data, uint32_t *smax, int32_t *sexp) {
+                                             int32_t stride, cx_t<T> *data, const S &slots) {
     using C = cx_t<T>;
-    for (int32_t l = t0; l < n_refs; l += stride) {
-        const LeafRef r = refs[l];
-        if (r.slot >= 0) {
-            smax[r.slot] = __ldcg(j.maxbits + r.node);
-            sexp[r.slot] = __ldcg(j.exp2 + r.node);
+    constexpr int LB = kStagePiece;
+#pragma unroll 1
+    for (int32_t l0 = 0; l0 < n_refs; l0 += stride) {
+        const int32_t l = l0 + t0;
+        LeafRef r;
+        r.count = 0;
+        if (l < n_refs) {
+            r = refs[l];
+            if (r.slot >= 0) slots.put(r.slot, __ldcg(j.maxbits + r.node), __ldcg(j.exp2 + r.node));
         }
         const C *src = (r.src ? reinterpret_cast<const C *>(j.arena) : static_cast<const C *>(j.leaf)) + r.global_off;
-        for (int32_t i0 = 0; i0 < r.count; i0 += LB) {
-            C v[LB];
+        C v[LB];
 #pragma unroll
-            for (int u = 0; u < LB; ++u)
-                if (i0 + u < r.count) v[u] = __ldcg(src + i0 + u);
+        for (int u = 0; u < LB; ++u)
+            if (u < r.count) v[u] = __ldcg(src + u);
 #pragma unroll
-            for (int u = 0; u < LB; ++u)
-                if (i0 + u < r.count) data[r.smem_off + i0 + u] = v[u];
-        }
+        for (int u = 0; u < LB; ++u)
+            if (u < r.count) data[r.smem_off + u] = v[u];
     }
 }
 
@@ -178,137 +186,202 @@ __device__ __forceinline__ void df_add(float &hi, float &lo, float xh, float xl)
     lo = __fadd_rn(lo, __fadd_rn(xl, t));
 }
 
-// A small step computed by one warp: C = A * B with A, B and C at any address (shared memory, or
-// global memory in warp programs).  S lanes share an output (S a power of two, S <= 32 / outputs,
-// S <= K) and split its shared index; their partial sums are combined with xor shuffles.  The
-// shared-index offsets are computed once per 32 indices -- lane l holds (kA, kB) of index k0 + l,
-// packed in 16 bits each (program operands have fewer than 2^16 elements) -- and are broadcast
-// with a shuffle.  The operand scales 2^-eA and 2^-eB are applied together on the B side when
-// their product is a normal number (products then round exactly as with separate scaling), else
-// separately.  In complex64 each output is accumulated as hi + lo pairs from exact products and
-// exact pairwise sums, and rounded once when it is stored: these steps are most of a circuit's
-// steps, and with plain FP32 multiply-adds their several roundings per output (rather than the one
-// of storing it) tripled the error of small amplitudes; the extra arithmetic costs about 3 % of
-// the time of a batch of 24-qubit brickwork amplitudes, where these steps are latency-bound.
-// Returns the warp-wide max-abs of C (every lane).
+// The sum of one output of a small step.  In complex64 Re and Im are kept as hi + lo pairs of exact
+// products and exact pairwise sums, rounded once when the output is stored: these steps are most of a
+// circuit's steps, and with plain FP32 multiply-adds their several roundings per output (rather than
+// the one of storing it) tripled the error of small amplitudes.
+template <typename T> struct SmallSum;
+template <> struct SmallSum<float> {
+    float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
+    __device__ __forceinline__ void mac(float2 a, float2 b) {
+        const float p1 = __fmul_rn(a.x, b.x), e1 = __fmaf_rn(a.x, b.x, -p1);
+        const float p2 = __fmul_rn(a.y, b.y), e2 = __fmaf_rn(a.y, b.y, -p2);
+        const float p3 = __fmul_rn(a.x, b.y), e3 = __fmaf_rn(a.x, b.y, -p3);
+        const float p4 = __fmul_rn(a.y, b.x), e4 = __fmaf_rn(a.y, b.x, -p4);
+        float s1, t1, s2, t2;
+        two_sum(p1, -p2, s1, t1);
+        two_sum(p3, p4, s2, t2);
+        df_add(rh, rl, s1, __fadd_rn(__fsub_rn(e1, e2), t1));
+        df_add(ih, il, s2, __fadd_rn(__fadd_rn(e3, e4), t2));
+    }
+    __device__ __forceinline__ void join(int32_t off) {
+        const float orh = __shfl_xor_sync(0xffffffffu, rh, off), orl = __shfl_xor_sync(0xffffffffu, rl, off);
+        const float oih = __shfl_xor_sync(0xffffffffu, ih, off), oil = __shfl_xor_sync(0xffffffffu, il, off);
+        df_add(rh, rl, orh, orl);
+        df_add(ih, il, oih, oil);
+    }
+    __device__ __forceinline__ float2 value() const { return cmake(__fadd_rn(rh, rl), __fadd_rn(ih, il)); }
+};
+template <> struct SmallSum<double> {
+    double2 acc = {0.0, 0.0};
+    __device__ __forceinline__ void mac(double2 a, double2 b) { cfma(acc, a, b); }
+    __device__ __forceinline__ void join(int32_t off) {
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
+    }
+    __device__ __forceinline__ double2 value() const { return acc; }
+};
+
+// One pass of a tabulated small step: NP outputs per lane group, with table words t[], their shared
+// index split over the S = 2^lg lanes of the group.  The sums of the NP outputs are independent chains.
+template <typename T, int NP>
+__device__ __forceinline__ float small_pass(const uint32_t *ktab, int32_t K, int32_t lg, int32_t sub,
+                                            const uint32_t (&t)[NP], const int32_t (&o)[NP], int32_t O,
+                                            const cx_t<T> *A, const cx_t<T> *B, cx_t<T> *Cp, bool fold, T sA, T sB) {
+    using C = cx_t<T>;
+    SmallSum<T> sum[NP];
+#pragma unroll 1
+    for (int32_t k0 = 0; k0 < K; k0 += 1 << lg) {
+        const int32_t k = k0 + sub;
+        const bool in = k < K;
+        const uint32_t p = ktab[in ? k : 0];
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            const uint32_t q = t[i] + p;   // both 16-bit offsets at once: neither overflows
+            C a = A[q & 0xffffu], b = B[q >> 16];
+            if (!fold) a = cscale(a, sA);
+            b = cscale(b, sB);
+            if (!in) a = b = cmake((T)0, (T)0);
+            sum[i].mac(a, b);
+        }
+    }
+    float mx = 0.f;
+    if (NP == 1) {   // two outputs per lane only come with whole shared indices
+#pragma unroll 1
+        for (int32_t off = (1 << lg) >> 1; off > 0; off >>= 1) sum[0].join(off);
+    }
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        const C v = sum[i].value();
+        if (o[i] < O && sub == 0) {
+            Cp[o[i]] = v;
+            mx = fmaxf(mx, absmax2(v));
+        }
+    }
+    return mx;
+}
+
+// A small step computed by `parts` warps, of which the calling one is `part`: C = A * B with A, B and
+// C at any address (shared memory, or global memory in warp programs).  S = 2^lg_split lanes share an
+// output and split its shared index; their partial sums are combined with xor shuffles.  The passes of
+// 32 / S outputs are dealt to the parts.  The operand scales 2^-eA and 2^-eB are applied together on
+// the B side when their product is a normal number (products then round exactly as with separate
+// scaling), else separately.
+// Bound by instruction issue in large batches and by the chain of dependent operations in small ones;
+// a lane therefore works on two outputs at a time where a step has them, and tabulated steps (all but
+// a few) spend three instructions per operand on addresses.  Measured against one output at a time and
+// tables for at most 16 outputs: the warp programs of 2432 24-qubit amplitudes 550 us (755 us), those
+// of 512 10-qubit amplitudes 57 us (77 us).  Steps without tables compute the
+// shared-index offsets once per 32 indices -- lane l holds (kA, kB) of index k0 + l, packed in 16 bits
+// each (program operands have fewer than 2^16 elements) -- and broadcast them with a shuffle.
+// Returns the warp-wide max-abs of its part of C (every lane).
 template <typename T>
 __device__ __forceinline__ float small_core(const LocalStep &s, const cx_t<T> *A, const cx_t<T> *B, cx_t<T> *Cp,
-                                            int32_t eA, int32_t eB) {
+                                            int32_t eA, int32_t eB, int32_t part, int32_t parts) {
     using C = cx_t<T>;
     const int lane = threadIdx.x & 31;
     const int32_t es = eA + eB;
     const bool fold = es > -120 && es < 120;
     const T sA = fold ? (T)1 : pow2<T>(-eA);
     const T sB = fold ? pow2<T>(-es) : pow2<T>(-eB);
-    const int32_t N = s.N, K = s.K, O = s.M * s.N;
-    const bool tab = (s.flags & LFLAG_TAB) != 0;
-    const uint32_t *tbl = reinterpret_cast<const uint32_t *>(reinterpret_cast<const char *>(&s) +
-                                                             offsetof(LocalStep, m_dim));
-    int32_t S = 1;
-    while (S * 2 * O <= 32 && S < K) S *= 2;
-    const int32_t sub = lane & (S - 1), per_pass = 32 / S;
-    const bool p2 = s.pow2;
+    const int32_t N = s.N, K = s.K, O = s.M * s.N, lg = s.lg_split;
+    const int32_t sub = lane & ((1 << lg) - 1), per_pass = 32 >> lg;
     float mx = 0.f;
-    for (int32_t o0 = 0; o0 < O; o0 += per_pass) {
-        const int32_t o = o0 + lane / S;
+    if (s.flags & LFLAG_TAB) {
+        const uint32_t *tbl = reinterpret_cast<const uint32_t *>(reinterpret_cast<const char *>(&s) +
+                                                                 offsetof(LocalStep, m_dim));
+        const uint32_t *ktab = tbl + kTabOut, *high = ktab + K;
+        auto word = [&](int32_t o) {   // idle lanes compute output 0 and store nothing
+            const int32_t i = o < O ? o : 0;
+            return O > kTabOut ? tbl[i & (kTabOut - 1)] + high[i / kTabOut] : tbl[i];
+        };
+        const int32_t stride = parts * per_pass;
+        int32_t o0 = part * per_pass;
+        if (lg == 0)
+#pragma unroll 1
+        for (; o0 + stride < O; o0 += 2 * stride) {
+            const int32_t o[2] = {o0 + (lane >> lg), o0 + stride + (lane >> lg)};
+            const uint32_t t[2] = {word(o[0]), word(o[1])};
+            mx = fmaxf(mx, small_pass<T, 2>(ktab, K, lg, sub, t, o, O, A, B, Cp, fold, sA, sB));
+        }
+        if (o0 < O) {
+            const int32_t o[1] = {o0 + (lane >> lg)};
+            const uint32_t t[1] = {word(o[0])};
+            mx = fmaxf(mx, small_pass<T, 1>(ktab, K, lg, sub, t, o, O, A, B, Cp, fold, sA, sB));
+        }
+        // non-negative floats order like their bit patterns
+        return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
+    }
+    const bool p2 = s.pow2;
+#pragma unroll 1
+    for (int32_t o0 = part * per_pass; o0 < O; o0 += parts * per_pass) {
+        const int32_t o = o0 + (lane >> lg);
         const bool act = o < O;
         int32_t oa = 0, ob = 0;
-        if (act && tab) {
-            const uint32_t t = tbl[o];
-            oa = (int32_t)(t & 0xffffu);
-            ob = (int32_t)(t >> 16);
-        } else if (act) {
+        if (act) {
             const int32_t m = o / N, n = o - m * N;
             oa = lgroup_off(s.nm, s.m_dim, s.m_str, s.m_lsb, p2, m);
             ob = lgroup_off(s.nn, s.n_dim, s.n_str, s.n_lsb, p2, n);
         }
-        C acc = cmake((T)0, (T)0);
-        float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;   // complex64: the sums as hi + lo pairs
+        SmallSum<T> sum;
+#pragma unroll 1
         for (int32_t k0 = 0; k0 < K; k0 += 32) {
             uint32_t packed = 0;
             if (k0 + lane < K) {
-                if (tab) {
-                    packed = tbl[kTabOut + lane];   // K <= kTabK: one pass, k0 = 0
-                } else {
-                    int32_t ka, kb;
-                    lgroup_off2(s, k0 + lane, ka, kb);
-                    packed = (uint32_t)ka | ((uint32_t)kb << 16);
-                }
+                int32_t ka, kb;
+                lgroup_off2(s, k0 + lane, ka, kb);
+                packed = (uint32_t)ka | ((uint32_t)kb << 16);
             }
             const int32_t kn = min(32, K - k0);
-            for (int32_t kk = 0; kk < kn; kk += S) {
+#pragma unroll 1
+            for (int32_t kk = 0; kk < kn; kk += 1 << lg) {
                 const int32_t k = kk + sub;
                 const uint32_t p = __shfl_sync(0xffffffffu, packed, k & 31);
                 if (act && k < kn) {
-                    const C a = A[oa + (int32_t)(p & 0xffffu)];
-                    const C b = B[ob + (int32_t)(p >> 16)];
-                    const C as = fold ? a : cscale(a, sA), bs = cscale(b, sB);
-                    if constexpr (sizeof(T) == 4) {
-                        // exact products, then exact sums of pairs: Re and Im of a * b as hi + lo
-                        const float p1 = __fmul_rn(as.x, bs.x), e1 = __fmaf_rn(as.x, bs.x, -p1);
-                        const float p2 = __fmul_rn(as.y, bs.y), e2 = __fmaf_rn(as.y, bs.y, -p2);
-                        const float p3 = __fmul_rn(as.x, bs.y), e3 = __fmaf_rn(as.x, bs.y, -p3);
-                        const float p4 = __fmul_rn(as.y, bs.x), e4 = __fmaf_rn(as.y, bs.x, -p4);
-                        float s1, t1, s2, t2;
-                        two_sum(p1, -p2, s1, t1);
-                        two_sum(p3, p4, s2, t2);
-                        df_add(rh, rl, s1, __fadd_rn(__fsub_rn(e1, e2), t1));
-                        df_add(ih, il, s2, __fadd_rn(__fadd_rn(e3, e4), t2));
-                    } else {
-                        cfma(acc, as, bs);
-                    }
+                    const C a = A[oa + (int32_t)(p & 0xffffu)], b = B[ob + (int32_t)(p >> 16)];
+                    sum.mac(fold ? a : cscale(a, sA), cscale(b, sB));
                 }
             }
         }
-        if constexpr (sizeof(T) == 4) {
-            for (int32_t off = S >> 1; off > 0; off >>= 1) {
-                const float orh = __shfl_xor_sync(0xffffffffu, rh, off), orl = __shfl_xor_sync(0xffffffffu, rl, off);
-                const float oih = __shfl_xor_sync(0xffffffffu, ih, off), oil = __shfl_xor_sync(0xffffffffu, il, off);
-                df_add(rh, rl, orh, orl);
-                df_add(ih, il, oih, oil);
-            }
-            acc = cmake(__fadd_rn(rh, rl), __fadd_rn(ih, il));   // one rounding of each sum
-        } else {
-            for (int32_t off = S >> 1; off > 0; off >>= 1) {
-                acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
-                acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
-            }
-        }
+#pragma unroll 1
+        for (int32_t off = (1 << lg) >> 1; off > 0; off >>= 1) sum.join(off);
+        const C v = sum.value();
         if (act && sub == 0) {
-            Cp[o] = acc;
-            mx = fmaxf(mx, absmax2(acc));
+            Cp[o] = v;
+            mx = fmaxf(mx, absmax2(v));
         }
     }
-    // non-negative floats order like their bit patterns
     return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
 }
 
-// A small step of a block program, run by one warp; the warp publishes the output's max-abs and
-// exponent itself.
+// A small step of a block program, run by `parts` warps; they publish the output's max-abs (the slot
+// starts at zero) and exponent themselves.
 template <typename T>
-__device__ __forceinline__ void local_small(const LocalStep &s, const LocalSmem &L) {
+__device__ __forceinline__ void local_small(const LocalStep &s, const LocalSmem &L, int32_t part, int32_t parts) {
     using C = cx_t<T>;
     const int32_t eA = scale_exponent(L.smax[s.sa]), eB = scale_exponent(L.smax[s.sb]);
     const float mx = small_core<T>(s, reinterpret_cast<const C *>(L.data) + s.a_off,
                                    reinterpret_cast<const C *>(L.data) + s.b_off,
-                                   reinterpret_cast<C *>(L.data) + s.c_off, eA, eB);
+                                   reinterpret_cast<C *>(L.data) + s.c_off, eA, eB, part, parts);
     if ((threadIdx.x & 31) == 0) {
-        L.smax[s.sc] = __float_as_uint(mx);
-        L.sexp[s.sc] = L.sexp[s.sa] + eA + L.sexp[s.sb] + eB;
+        if (parts > 1) atomicMax(L.smax + s.sc, __float_as_uint(mx));
+        else L.smax[s.sc] = __float_as_uint(mx);
+        if (part == 0) L.sexp[s.sc] = L.sexp[s.sa] + eA + L.sexp[s.sb] + eB;
     }
 }
 
-// Shared-memory slice of a warp program: the current step's descriptor, the scale slots of its
-// intermediates, then the intermediates (the host computes the same sizes).
+// Shared-memory slice of a warp program: the descriptors of the current and the next step, the scale
+// slots {max-abs bits, exponent} of its nodes, then the leaves and intermediates (the host computes
+// the same sizes).
 __device__ __host__ __forceinline__ size_t warp_fixed_bytes(int32_t n_slots) {
-    return sizeof(LocalStep) + ((8 * (size_t)n_slots + 15) / 16) * 16;
+    return 2 * sizeof(LocalStep) + ((8 * (size_t)n_slots + 15) / 16) * 16;
 }
 
 // Runs warp program `prog` of job `j` in the calling warp, `slice` being its kWarpSlice bytes of
 // shared memory.  The warp stages the program's leaves into the slice, then runs the steps in
 // plan order with every operand in shared memory; the last step writes the program's result (and
-// its max-abs and exponent) to global memory.  Each step's descriptor is prefetched while the
-// previous step runs.
+// its max-abs and exponent) to global memory.  Descriptors are fetched two steps ahead, so that a
+// step does not wait for the L2 round trip of the next one's.
 template <typename T>
 __device__ void run_warp_prog(int32_t prog, const JobPtrs &j, char *slice) {
     using C = cx_t<T>;
@@ -317,34 +390,38 @@ __device__ void run_warp_prog(int32_t prog, const JobPtrs &j, char *slice) {
     const int32_t n_steps = P.n_steps, first = P.first_step, n_slots = P.n_slots;
     const int64_t root_c_off = P.root_c_off;
     const int32_t root_node = P.root_node;
-    LocalStep *desc = reinterpret_cast<LocalStep *>(slice);
-    uint32_t *smax = reinterpret_cast<uint32_t *>(slice + sizeof(LocalStep));
-    int32_t *sexp = reinterpret_cast<int32_t *>(smax + n_slots);
+    int2 *slot = reinterpret_cast<int2 *>(slice + 2 * sizeof(LocalStep));
     C *data = reinterpret_cast<C *>(slice + warp_fixed_bytes(n_slots));
     constexpr int kPieces = (int)(sizeof(LocalStep) / sizeof(int4));
     static_assert(kPieces <= 32, "one descriptor piece per lane");
     const int4 *dsrc = reinterpret_cast<const int4 *>(j.lsteps + first);
-    int4 nxt = make_int4(0, 0, 0, 0);
-    if (lane < kPieces) nxt = __ldg(dsrc + lane);
-    stage_inputs<T>(j, j.leafrefs + P.first_leaf, P.n_leaves, lane, 32, data, smax, sexp);
+    auto fetch = [&](int32_t si) {
+        return lane < kPieces && si < n_steps ? __ldg(dsrc + (int64_t)si * kPieces + lane) : make_int4(0, 0, 0, 0);
+    };
+    auto put = [&](int32_t si, const int4 &d) {
+        if (lane < kPieces) reinterpret_cast<int4 *>(slice + (si & 1) * sizeof(LocalStep))[lane] = d;
+    };
+    const int4 d0 = fetch(0);
+    int4 nxt = fetch(1);
+    stage_inputs<T>(j, j.leafrefs + P.first_leaf, P.n_leaves, lane, 32, data, PairSlots{slot});
+    put(0, d0);
     for (int32_t si = 0; si < n_steps; ++si) {
-        __syncwarp();   // staging / the previous step are done with the slice and the descriptor
-        if (lane < kPieces) reinterpret_cast<int4 *>(desc)[lane] = nxt;
-        __syncwarp();
-        if (si + 1 < n_steps && lane < kPieces) nxt = __ldg(dsrc + (int64_t)(si + 1) * kPieces + lane);
-        const LocalStep &s = *desc;
-        const int32_t eA = scale_exponent(smax[s.sa]), eB = scale_exponent(smax[s.sb]);
-        const int32_t e = sexp[s.sa] + eA + sexp[s.sb] + eB;
+        __syncwarp();   // staging / the previous step are done, its descriptor's place is free
+        put(si + 1, nxt);
+        nxt = fetch(si + 2);
+        const LocalStep &s = *reinterpret_cast<const LocalStep *>(slice + (si & 1) * sizeof(LocalStep));
+        const int2 ma = slot[s.sa], mb = slot[s.sb];
+        const int32_t eA = scale_exponent((uint32_t)ma.x), eB = scale_exponent((uint32_t)mb.x);
+        const int32_t e = ma.y + eA + mb.y + eB;
         const bool out = s.flags & LFLAG_C_OUT;
         C *Cp = out ? reinterpret_cast<C *>(j.arena) + root_c_off : data + s.c_off;
-        const float mx = small_core<T>(s, data + s.a_off, data + s.b_off, Cp, eA, eB);
+        const float mx = small_core<T>(s, data + s.a_off, data + s.b_off, Cp, eA, eB, 0, 1);
         if (lane == 0) {
             if (out) {
                 j.maxbits[root_node] = __float_as_uint(mx);
                 j.exp2[root_node] = e;
             } else {
-                smax[s.sc] = __float_as_uint(mx);
-                sexp[s.sc] = e;
+                slot[s.sc] = make_int2((int32_t)__float_as_uint(mx), e);
             }
         }
     }
@@ -685,7 +762,8 @@ __device__ void run_local(int32_t prog, const JobPtrs &j, char *dyn, char *scrat
     }
     for (int32_t i = threadIdx.x; i < P.n_slots; i += blockDim.x) { L.smax[i] = 0u; L.sexp[i] = 0; }
     __syncthreads();
-    stage_inputs<T>(j, j.leafrefs + P.first_leaf, P.n_leaves, threadIdx.x, blockDim.x, data, L.smax, L.sexp);
+    stage_inputs<T>(j, j.leafrefs + P.first_leaf, P.n_leaves, threadIdx.x, blockDim.x, data,
+                    SplitSlots{L.smax, L.sexp});
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     __syncthreads();
     long long tp = 0;
@@ -715,8 +793,12 @@ __device__ void run_local(int32_t prog, const JobPtrs &j, char *dyn, char *scrat
                 atomicAdd((unsigned long long *)(prof + kProfSlots + 14), 1ull);
             }
         }
-        // independent small steps: one warp each
-        for (int32_t i = warp; i < W.n_small; i += nw) local_small<T>(L.desc[W.first + i], L);
+        // independent small steps: one warp each, or several when there are fewer steps than warps (a
+        // step of 256 outputs and 16 shared indices takes one warp 13000 cycles; the block programs of
+        // 512 10-qubit amplitudes took 82 us with one warp per step and take 37 us)
+        const int32_t parts = W.n_small > 0 && W.n_small < nw ? nw / W.n_small : 1;
+        for (int32_t i = warp / parts; i < W.n_small; i += nw / parts)
+            local_small<T>(L.desc[W.first + i], L, warp % parts, parts);
         // big steps: the whole block, one after the other
         for (int32_t i = 0; i < W.n_big; ++i) {
             const LocalStep &s = L.desc[W.first + W.n_small + i];

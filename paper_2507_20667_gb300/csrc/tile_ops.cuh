@@ -57,38 +57,55 @@ template <> __device__ __forceinline__ double pow2<double>(int32_t e) {
 __device__ __forceinline__ float absmax2(float2 v) { return fmaxf(fabsf(v.x), fabsf(v.y)); }
 __device__ __forceinline__ float absmax2(double2 v) { return (float)fmax(fabs(v.x), fabs(v.y)); }
 
+// Digits by division (dims that are not powers of two), kept out of line: inlined at each of its
+// uses in every tile shape, the 64-bit divisions were most of the kernels' code (k_persist 1.2 MB),
+// which does not stay in the instruction caches.
+static __device__ __noinline__ int64_t group_off_div(const Groups *g, int64_t idx) {
+    int64_t off = 0;
+#pragma unroll 1
+    for (int32_t i = 0; i < g->n; ++i) {
+        const int64_t q = idx / g->dim[i];
+        off += (idx - q * g->dim[i]) * g->sa[i];
+        idx = q;
+    }
+    return off;
+}
+static __device__ __noinline__ longlong2 group_off2_div(const Groups *g, int64_t idx) {
+    longlong2 off = make_longlong2(0, 0);
+#pragma unroll 1
+    for (int32_t i = 0; i < g->n; ++i) {
+        const int64_t q = idx / g->dim[i], d = idx - q * g->dim[i];
+        off.x += d * g->sa[i];
+        off.y += d * g->sb[i];
+        idx = q;
+    }
+    return off;
+}
+
 // Offset contributed by the digits of `idx` over a group list (stride `sa`).
 __device__ __forceinline__ int64_t group_off(const Groups &g, int64_t idx) {
+    if (!g.pow2) return group_off_div(&g, idx);
     int64_t off = 0;
-    if (g.pow2) {
-        for (int32_t i = 0; i < g.n; ++i) off += ((idx >> g.lsb[i]) & g.mask[i]) * g.sa[i];
-    } else {
-        for (int32_t i = 0; i < g.n; ++i) {
-            int64_t d = idx % g.dim[i];
-            idx /= g.dim[i];
-            off += d * g.sa[i];
-        }
-    }
+#pragma unroll 4
+    for (int32_t i = 0; i < g.n; ++i) off += ((idx >> g.lsb[i]) & g.mask[i]) * g.sa[i];
     return off;
 }
 
 // Offsets in A and B of a shared-leg multi-index.
 __device__ __forceinline__ void group_off2(const Groups &g, int64_t idx, int64_t &oa, int64_t &ob) {
+    if (!g.pow2) {
+        const longlong2 o = group_off2_div(&g, idx);
+        oa = o.x;
+        ob = o.y;
+        return;
+    }
     oa = 0;
     ob = 0;
-    if (g.pow2) {
-        for (int32_t i = 0; i < g.n; ++i) {
-            int64_t d = (idx >> g.lsb[i]) & g.mask[i];
-            oa += d * g.sa[i];
-            ob += d * g.sb[i];
-        }
-    } else {
-        for (int32_t i = 0; i < g.n; ++i) {
-            int64_t d = idx % g.dim[i];
-            idx /= g.dim[i];
-            oa += d * g.sa[i];
-            ob += d * g.sb[i];
-        }
+#pragma unroll 4
+    for (int32_t i = 0; i < g.n; ++i) {
+        const int64_t d = (idx >> g.lsb[i]) & g.mask[i];
+        oa += d * g.sa[i];
+        ob += d * g.sb[i];
     }
 }
 

@@ -347,3 +347,48 @@ def test_large_leaves_max_abs_across_slices(tnsa, ctx, prec):
     ref = np.dot(down(us), down(vs))
     got = complex(np.ldexp(m.real, int(e) - 2 * big), np.ldexp(m.imag, int(e) - 2 * big))
     check(got, ref, TOL[prec], f"{prec} dot of {L} entries")
+
+
+# small steps: (free legs of A, shared legs, free legs of B) -- one pass or several, shared indices split
+# over lanes or not, tabulated index maps (up to 256 outputs) or decoded ones, dims that are no powers of two
+@pytest.mark.parametrize("legs", [((2,), (2,), ()), ((2, 2), (2,), (2, 2)), ((2,) * 3, (2,) * 4, (2,)),
+                                  ((2,) * 4, (2,) * 3, (2,) * 4), ((2,) * 4, (2,) * 4, (2,) * 4), ((), (2,) * 6, (2,)),
+                                  ((2,) * 5, (2,), ()), ((4, 8), (2, 4), (4,)), ((3,), (3,), (2,)), ((5,), (3, 2), (3,)),
+                                  ((3, 7), (2,), (5,)), ((2, 8), (1,), (2, 4))])
+@pytest.mark.parametrize("precision", ["c64", "c128"])
+def test_small_step_shapes(tnsa, legs, precision):
+    fa, sh, fb = legs
+    rng = np.random.default_rng(len(fa) * 100 + len(sh) * 10 + len(fb))
+    names = iter("abcdefghijklmnopqrstuvwxyz")
+    la, ls, lb = [[next(names) for _ in x] for x in legs]
+    dim = dict(zip(la + ls + lb, fa + sh + fb))
+    # the legs of each operand in an order of their own
+    axes = [list(rng.permutation(x)) for x in (la + ls, ls + lb, la + lb)]
+    tensors = [rng.standard_normal([dim[i] for i in x]) + 1j * rng.standard_normal([dim[i] for i in x]) for x in axes]
+    where = {}
+    for t, x in enumerate(axes):
+        for i, name in enumerate(x):
+            where.setdefault(name, []).extend((t, i))
+    net = tni.Network([np.ascontiguousarray(t) for t in tensors], np.array(list(where.values()), np.int32).reshape(-1, 4),
+                         np.zeros(3, np.int32), ["t"] * 3)
+    h = tnsa.tn_build(net)
+    plan = tnsa.tn_plan_import(h, [(0, 1), (3, 2)])
+    m, e, _ = tnsa.tn_contract(tnsa.tn_ctx_create(0), h, plan, precision)
+    spec = ",".join("".join(x) for x in axes) + "->"
+    ref, scale = np.einsum(spec, *tensors), np.einsum(spec, *(np.abs(t) for t in tensors))
+    # each factor is rounded once, so are the step's outputs and the closing products
+    assert abs(m * 2.0 ** e - ref) <= 8 * (2.0 ** -24 if precision == "c64" else 2.0 ** -53 * sum(map(len, axes))) * scale
+
+
+@pytest.mark.parametrize("length", [32, 33, 70])
+def test_warp_program_with_many_leaves(tnsa, length):
+    """A closed chain of 2 x 2 matrices: one warp program with more staging pieces than lanes."""
+    rng = np.random.default_rng(length)
+    mats = [np.linalg.qr(rng.standard_normal((2, 2)) + 1j * rng.standard_normal((2, 2)))[0] for _ in range(length)]
+    edges = [(i, 1, (i + 1) % length, 0) for i in range(length)]
+    net = tni.Network(mats, np.array(edges, np.int32), np.zeros(length, np.int32), ["t"] * length)
+    h = tnsa.tn_build(net)
+    steps = [(0, 1)] + [(length + i - 2, i) for i in range(2, length)]
+    m, e, _ = tnsa.tn_contract(tnsa.tn_ctx_create(0), h, tnsa.tn_plan_import(h, steps), "c64")
+    # unitary factors: every rounding adds at most 2^-24 of the norm of a 2 x 2 block, twice per factor
+    assert abs(m * 2.0 ** e - np.trace(np.linalg.multi_dot(mats))) <= 4 * length * 2.0 ** -24
