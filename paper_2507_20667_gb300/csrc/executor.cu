@@ -817,8 +817,9 @@ tn_status tn::compile(Compiled &c, const Net &net, const Plan &plan, const Compi
             p.part_off = (int32_t)c.n_partials;
             c.n_partials += (int64_t)p.ntiles * kDotMaxOut;
             // tabulate the shared-index offsets (the tile then reads one int2 per index instead of
-            // decomposing the index over its leg groups) when the table stays small
-            if (K <= (1 << 20)) {
+            // decomposing the index over its leg groups) when the table stays small; one fused group
+            // needs no table
+            if (K <= (1 << 20) && p.k.n != 1) {
                 bool fits = true;
                 const size_t t0 = c.ktab.size();
                 c.ktab.resize(t0 + (size_t)K);

@@ -392,3 +392,34 @@ def test_warp_program_with_many_leaves(tnsa, length):
     m, e, _ = tnsa.tn_contract(tnsa.tn_ctx_create(0), h, tnsa.tn_plan_import(h, steps), "c64")
     # unitary factors: every rounding adds at most 2^-24 of the norm of a 2 x 2 block, twice per factor
     assert abs(m * 2.0 ** e - np.trace(np.linalg.multi_dot(mats))) <= 4 * length * 2.0 ** -24
+
+
+# closing dots on the dataflow path: lengths around the burst and tile sizes, both operands contiguous (with
+# and without 16-byte alignment: a first pair of `shift` entries moves the others) or one of them transposed
+@pytest.mark.parametrize("dims", [(1,), (7,), (511,), (4097,), (8191,), (8193,), (100001,), (130, 200), (64, 257, 3)])
+@pytest.mark.parametrize("shift", [2, 3])
+@pytest.mark.parametrize("transposed", [False, True])
+@pytest.mark.parametrize("precision", ["c64", "c128"])
+def test_long_dots(tnsa, dims, shift, transposed, precision):
+    if transposed and len(dims) == 1:
+        pytest.skip("one leg has one order")
+    rng = np.random.default_rng(len(dims) * 10 + shift)
+
+    def normal(*shape):
+        return rng.standard_normal(shape) + 1j * rng.standard_normal(shape)
+    a, b = normal(*dims), normal(*(dims[::-1] if transposed else dims))
+    p, q = normal(shift), normal(shift)
+    n = len(dims)
+    edges = [(0, 0, 1, 0)] + [(2, i, 3, n - 1 - i if transposed else i) for i in range(n)]
+    net = tni.Network([p, q, a, b], np.array(edges, np.int32), np.zeros(4, np.int32), ["t"] * 4)
+    h = tnsa.tn_build(net)
+    plan = tnsa.tn_plan_import(h, [(2, 3), (0, 1), (4, 5)])
+    c = tnsa.tn_ctx_create(0)
+    tnsa.tn_ctx_set_local_budget(c, 0)
+    m, e, _ = tnsa.tn_contract(c, h, plan, precision)
+    bt = b.transpose() if transposed else b
+    ref, scale = (a * bt).sum() * (p * q).sum(), np.abs(a * bt).sum() * np.abs(p * q).sum()
+    # complex64: leaves, products, sums of 8 products and the two stored dots are rounded (16 roundings at
+    # most on the way of a term); complex128: 8 products and then a sum per burst
+    eps = 16 * 2.0 ** -24 if precision == "c64" else (64 + math.prod(dims) / 2048) * 2.0 ** -53
+    assert abs(m * 2.0 ** e - ref) <= 2 * eps * scale
