@@ -289,6 +289,53 @@ int32_t rows_per_tile(int64_t M) {
     return 4096;
 }
 
+// The thread tile of a step staged whole through shared memory: the smallest one whose threads cover M
+// rows and N columns (-1: none, or the operands do not fit).  The limits are the kernel's: kRowsMaxK
+// table entries, A and then C in kRowsSmemElems elements, B in the scratch area or behind A.
+int32_t rows_shape(int64_t M, int64_t N, int64_t K) {
+    if (N > kRowsSmemN || K > kRowsMaxK || M * K > kRowsSmemElems || M * N > kRowsSmemElems) return -1;
+    for (int32_t s = 0; s < kRowsShapes; ++s) {
+        const int64_t groups = rows_groups(N, rows_nc(s));
+        if (M > kThreads / groups * rows_r(s)) continue;
+        const int64_t b = K * groups * rows_nc(s) * 8;
+        if (b <= Scratch<float>::bytes - kRowsTabBytes || align_up((size_t)(M * K * 8), 16) + b <= kRowsSmemElems * 8)
+            return s;
+    }
+    return -1;
+}
+
+// The offset table of a staged step, appended to `out`: byte offsets in A of the rows and of the shared
+// indices (swizzled for power-of-two dims), then element offsets in B -- of each (shared index, column of
+// the thread tiles), -1 past the columns, or for small steps of the shared indices and of the columns.
+void staged_table(const StepDesc &d, std::vector<int2> &out) {
+    auto dec = [](const Groups &g, int64_t idx, const int64_t *str) {
+        int64_t off = 0;
+        for (int32_t i = 0; i < g.n; ++i) {
+            off += idx % g.dim[i] * str[i];
+            idx /= g.dim[i];
+        }
+        return off;
+    };
+    const bool p2 = d.m.pow2 && d.k.pow2;
+    std::vector<int32_t> t;
+    auto a_bytes = [&](int64_t o) { t.push_back((int32_t)(8 * (p2 ? swz((uint32_t)o) : (uint32_t)o))); };
+    for (int64_t m = 0; m < d.M; ++m) a_bytes(dec(d.m, m, d.m.sa));
+    for (int64_t k = 0; k < d.K; ++k) a_bytes(dec(d.k, k, d.k.sa));
+    std::vector<int32_t> kb(d.K), nb(d.N);
+    for (int64_t k = 0; k < d.K; ++k) kb[k] = (int32_t)dec(d.k, k, d.k.sb);
+    for (int64_t n = 0; n < d.N; ++n) nb[n] = (int32_t)dec(d.n, n, d.n.sa);
+    if (d.tile_shape == kRowsShapeSmall) {
+        t.insert(t.end(), kb.begin(), kb.end());
+        t.insert(t.end(), nb.begin(), nb.end());
+    } else {
+        const int32_t NB = rows_groups(d.N, rows_nc(d.tile_shape)) * rows_nc(d.tile_shape);
+        for (int64_t k = 0; k < d.K; ++k)
+            for (int32_t n = 0; n < NB; ++n) t.push_back(n < d.N ? kb[k] + nb[n] : -1);
+    }
+    if (t.size() & 1) t.push_back(0);
+    for (size_t i = 0; i < t.size(); i += 2) out.push_back(make_int2(t[i], t[i + 1]));
+}
+
 // Geometry of one pairwise step: which child plays A (the larger), the free / shared legs with
 // their strides (outermost first), and M, N, K.
 struct Geom {
@@ -808,6 +855,8 @@ tn_status tn::compile(Compiled &c, const Net &net, const Plan &plan, const Compi
         d.level = 1 + std::max(level[g.a], level[g.b]);
         const int64_t M = g.M, N = g.N, K = g.K;
         const bool dot = root || (M * N <= kDotMaxOut && K > kRowsMaxK);
+        const bool dense = use_tc && M >= opt.tc_min_m && N >= opt.tc_min_n && K >= opt.tc_min_k &&
+                           !(N <= kRowsMaxN && K <= kRowsMaxK && K * N <= kRowsMaxKN);   // tensor cores
         if (dot) {
             StepDesc p = d;
             p.kind = STEP_DOTP;
@@ -862,22 +911,33 @@ tn_status tn::compile(Compiled &c, const Net &net, const Plan &plan, const Compi
             if (root) f.flags |= FLAG_ROOT | FLAG_NO_C;
             c.steps.push_back(f);
             c.counts[STEP_DOTP]++;
+        } else if (const int32_t shape = elem == 8 && !(d.flags & FLAG_A_LEAF) && !dense ? rows_shape(M, N, K) : -1;
+                   shape >= 0 && c.ktab.size() < 0x40000000) {
+            // complex64 steps that fit shared memory are staged through it whole; small ones are summed
+            // as the programs do
+            d.kind = STEP_ROWS;
+            d.flags |= FLAG_A_SMEM | (d.m.pow2 && d.k.pow2 ? FLAG_A_POW2 : 0);
+            d.tile_shape = small_step(g, root) ? kRowsShapeSmall : shape;
+            d.tile_rows = (int32_t)M;
+            d.ntiles = 1;
+            d.ktab_off = (int32_t)c.ktab.size();
+            staged_table(d, c.ktab);
+            c.steps.push_back(d);
+            c.counts[STEP_ROWS]++;
+        } else if (elem == 8 && !dense && small_step(g, root)) {
+            d.kind = STEP_ROWS;
+            d.flags |= FLAG_SMALL;
+            d.tile_rows = (int32_t)M;
+            d.ntiles = 1;
+            c.steps.push_back(d);
+            c.counts[STEP_ROWS]++;
         } else if (N <= kRowsMaxN && K <= kRowsMaxK && K * N <= kRowsMaxKN) {
             d.kind = STEP_ROWS;
             d.tile_rows = rows_per_tile(M);
             d.ntiles = (int32_t)((M + d.tile_rows - 1) / d.tile_rows);
-            // complex64 steps whose A fits shared memory are staged through it (one tile, every
-            // thread owning 32 / NT rows in one pass)
-            const int64_t nt = N <= 4 ? 4 : (N <= 8 ? 8 : 16);
-            if (elem == 8 && K <= 16 && !(d.flags & FLAG_A_LEAF) && M * K <= kRowsSmemElems &&
-                M * (N + 1) <= kRowsSmemElems && M <= (int64_t)kThreads * (32 / nt)) {
-                d.flags |= FLAG_A_SMEM;
-                d.tile_rows = (int32_t)M;
-                d.ntiles = 1;
-            }
             c.steps.push_back(d);
             c.counts[STEP_ROWS]++;
-        } else if (use_tc && M >= opt.tc_min_m && N >= opt.tc_min_n && K >= opt.tc_min_k) {
+        } else if (dense) {
             // dense step on the tensor cores: operands packed into split images, then 128 x 128
             // complex output tiles, BF16 or TF32 split
             d.kind = STEP_TC;
@@ -909,9 +969,9 @@ tn_status tn::compile(Compiled &c, const Net &net, const Plan &plan, const Compi
         level[o] = c.steps.back().level;
     }
     // ROWS chains: step t continues step s in the same persistent block, with s's C kept in
-    // shared memory as t's A, when both stage A through shared memory, A of t is C of s (its only
-    // consumer: the plan is a tree), N of s is a power of two (C's rotated layout) and B of t is a
-    // leaf or a program output (complete before the dataflow launch, so the chain never waits
+    // shared memory as t's A, when both are staged through shared memory, A of t is C of s (its only
+    // consumer: the plan is a tree), the dims of A are powers of two (C's swizzled layout) and B of t is
+    // a leaf or a program output (complete before the dataflow launch, so the chain never waits
     // inside).  Steps are in plan order, so s precedes t.
     if (opt.rows_chains) {
         std::vector<int32_t> chain_len(c.steps.size(), 1);
@@ -921,14 +981,11 @@ tn_status tn::compile(Compiled &c, const Net &net, const Plan &plan, const Compi
             StepDesc &s = c.steps[t.dep0];
             if (s.kind != STEP_ROWS || !(s.flags & FLAG_A_SMEM) || s.chain_next >= 0 || s.node_c != t.node_a)
                 continue;
-            if ((s.N & (s.N - 1)) != 0 || s.M * s.N != t.M * t.K) continue;
+            if (s.M * s.N != t.M * t.K || !t.m.pow2 || !t.k.pow2) continue;   // C is kept swizzled
             if (t.dep1 >= 0 && c.steps[t.dep1].kind != STEP_LOCAL) continue;
             if (chain_len[t.dep0] >= kMaxChain) continue;
             s.chain_next = (int32_t)ti;
             t.flags |= FLAG_CHAIN_CONT;
-            int32_t lg = 0;
-            while ((1LL << lg) < s.N) ++lg;
-            t.a_lgn = lg;
             chain_len[ti] = chain_len[t.dep0] + 1;
         }
     }

@@ -39,17 +39,20 @@ enum StepFlags : int32_t {
     FLAG_ROOT = 4,      // the step produces the network's value: write the job's result record
     FLAG_NO_C = 8,      // no tensor output (DOTP, or the root's DOTF)
     FLAG_TF32 = 16,     // TC: TF32 split (else BF16 split)
-    FLAG_A_SMEM = 32,   // ROWS: A is copied whole into shared memory and C leaves through it
+    FLAG_A_SMEM = 32,   // ROWS: the step is staged whole through shared memory (thread tile tile_shape)
     FLAG_CHAIN_CONT = 64, // ROWS (FLAG_A_SMEM): A is the C of the previous step of a chain, which
                           // the persistent kernel keeps in shared memory; no work item of its own
     FLAG_A_MCONT = 128,   // TC: A's row index is its contiguous one (the pack reads rows fastest)
     FLAG_B_NCONT = 256,   // TC: B's column index is its contiguous one
     FLAG_DOT_SMEM_A = 512,  // DOTP (complex64, one tile, M = 1): A, read in a permuted order, is
                             // first copied whole and coalesced into shared memory
-    FLAG_DOT_SMEM_B = 1024  // the same for B (N = 1)
+    FLAG_DOT_SMEM_B = 1024, // the same for B (N = 1)
+    FLAG_SMALL = 2048,      // ROWS: a small step (complex64), summed as in the subtree programs
+    FLAG_A_POW2 = 4096      // FLAG_A_SMEM: A's dims are powers of two (swizzled layout)
 };
 
-struct StepDesc {
+// The part of a step descriptor that staged steps need: their index maps are tabulated.
+struct StepHead {
     int64_t M, N, K;
     int64_t a_off, b_off, c_off;   // element offsets into the leaf buffer or the arena
     int64_t img_a, img_b;          // TC: byte offsets in the arena of the packed operand images
@@ -62,12 +65,18 @@ struct StepDesc {
                                    // TILE: tile shape (0: 64 x 64, kTileNarrow: 128 x 32)
     int32_t part_off;              // DOTP / DOTF: offset of the step's partials (in double2)
     int32_t level;                 // longest path from the leaves (scheduling order)
-    int32_t ktab_off;              // DOTP: first entry of its shared-index offset table (-1: none)
+    int32_t ktab_off;              // DOTP: first entry of its shared-index offset table (-1: none);
+                                   // FLAG_A_SMEM: of its table of A and B offsets (as int32)
     int32_t chain_next;            // ROWS (FLAG_A_SMEM): the step that consumes C next in the same
                                    // block, C kept in shared memory (-1: C goes to the arena)
-    int32_t a_lgn;                 // FLAG_CHAIN_CONT: log2 of the previous step's N (the row width
-                                   // of A's rotated shared-memory layout)
+    int32_t tile_shape;            // FLAG_A_SMEM: the thread tile, rows_shape()
+    int32_t pad[2];
+};
+static_assert(sizeof(StepHead) % 16 == 0, "heads are copied in 16-byte pieces");
+
+struct StepDesc : StepHead {
     Groups m, n, k;
+    int64_t pad2;
 };
 
 // ---- CTA-resident subtree programs -------------------------------------------------------------
@@ -158,7 +167,8 @@ struct JobPtrs {
     const LocalStep *lsteps;
     const LeafRef *leafrefs;
     const LocalWave *lwaves;
-    const int2 *ktab;        // (offset in A, offset in B) of each shared index of tabulated DOTP steps
+    const int2 *ktab;        // (offset in A, offset in B) of each shared index of tabulated DOTP steps,
+                             // and the int32 tables of staged steps
     int32_t n_steps;
     int32_t n_leaves;
 };
@@ -245,10 +255,25 @@ constexpr int kTileM = 64, kTileN = 64, kTileK = 16;   // CUDA-core GEMM tile
 constexpr int kTileNarrow = 1;                          // TILE: tile_rows = 1 selects 128 x 32 tiles
 constexpr int kRowsMaxKN = 1024, kRowsMaxK = 64, kRowsMaxN = 16;
 constexpr int kDotMaxOut = 4;
-// ROWS steps staged through shared memory (complex64): A (M K elements) and then the padded C
-// (M (N + 1) elements) share kRowsSmemElems elements of the dataflow kernel's dynamic shared memory.
+// Steps staged whole through shared memory (complex64): A (M K elements), B where it does not fit the
+// scratch area and then C (M N elements) share kRowsSmemElems elements of the dataflow
+// kernel's dynamic shared memory; the A offsets of the shared indices take kRowsTabBytes.
 constexpr int kRowsSmemElems = 9216;
-constexpr int kPersistDynSmem = kRowsSmemElems * 8;
+constexpr int kRowsSmemN = 64;                          // most columns of a staged step
+constexpr int kRowsTabBytes = 64 * 4;
+// Thread tiles of staged steps, by increasing size: columns and rows per thread.  The columns are cut
+// into groups, a power of two of them; the kThreads / groups threads of a group share the rows.
+constexpr int kRowsShapes = 4, kRowsShapeSmall = 4;   // the last: small steps, an output per thread
+__host__ __device__ constexpr int rows_nc(int shape) { return shape == 2 ? 8 : 4; }
+__host__ __device__ constexpr int rows_r(int shape) { return shape == 0 ? 2 : shape == 3 ? 8 : 4; }
+__host__ __device__ constexpr int rows_groups(int64_t N, int nc) {
+    int g = 1;
+    while ((int64_t)g * nc < N) g *= 2;
+    return g;
+}
+// In a chain the next step's B is fetched ahead, up to kRowsAhead entries, behind that area.
+constexpr int kRowsAhead = 1024;
+constexpr int kPersistDynSmem = (kRowsSmemElems + kRowsAhead) * 8;
 // Longest chain of ROWS steps one persistent block runs with the tensor kept in shared memory.
 constexpr int kMaxChain = 32;
 constexpr int kDotChunk = 8192;                         // shared indices per DOTP tile

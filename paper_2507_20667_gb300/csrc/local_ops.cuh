@@ -169,59 +169,6 @@ __device__ __forceinline__ void stage_inputs_async(const JobPtrs &j, const LeafR
     }
 }
 
-// Error-free transformations (Knuth's TwoSum; the FMA form of Dekker's TwoProduct, as used by
-// Ogita, Rump and Oishi for accurate dot products), written with round-to-nearest intrinsics so
-// that the compiler neither contracts nor reorders them: a + b = s + err and a * b = p + err
-// exactly.
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &err) {
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-// A sum kept as an unevaluated pair hi + lo (about 44 significant bits); adds x = xh + xl.
-__device__ __forceinline__ void df_add(float &hi, float &lo, float xh, float xl) {
-    float s, t;
-    two_sum(hi, xh, s, t);
-    hi = s;
-    lo = __fadd_rn(lo, __fadd_rn(xl, t));
-}
-
-// The sum of one output of a small step.  In complex64 Re and Im are kept as hi + lo pairs of exact
-// products and exact pairwise sums, rounded once when the output is stored: these steps are most of a
-// circuit's steps, and with plain FP32 multiply-adds their several roundings per output (rather than
-// the one of storing it) tripled the error of small amplitudes.
-template <typename T> struct SmallSum;
-template <> struct SmallSum<float> {
-    float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-    __device__ __forceinline__ void mac(float2 a, float2 b) {
-        const float p1 = __fmul_rn(a.x, b.x), e1 = __fmaf_rn(a.x, b.x, -p1);
-        const float p2 = __fmul_rn(a.y, b.y), e2 = __fmaf_rn(a.y, b.y, -p2);
-        const float p3 = __fmul_rn(a.x, b.y), e3 = __fmaf_rn(a.x, b.y, -p3);
-        const float p4 = __fmul_rn(a.y, b.x), e4 = __fmaf_rn(a.y, b.x, -p4);
-        float s1, t1, s2, t2;
-        two_sum(p1, -p2, s1, t1);
-        two_sum(p3, p4, s2, t2);
-        df_add(rh, rl, s1, __fadd_rn(__fsub_rn(e1, e2), t1));
-        df_add(ih, il, s2, __fadd_rn(__fadd_rn(e3, e4), t2));
-    }
-    __device__ __forceinline__ void join(int32_t off) {
-        const float orh = __shfl_xor_sync(0xffffffffu, rh, off), orl = __shfl_xor_sync(0xffffffffu, rl, off);
-        const float oih = __shfl_xor_sync(0xffffffffu, ih, off), oil = __shfl_xor_sync(0xffffffffu, il, off);
-        df_add(rh, rl, orh, orl);
-        df_add(ih, il, oih, oil);
-    }
-    __device__ __forceinline__ float2 value() const { return cmake(__fadd_rn(rh, rl), __fadd_rn(ih, il)); }
-};
-template <> struct SmallSum<double> {
-    double2 acc = {0.0, 0.0};
-    __device__ __forceinline__ void mac(double2 a, double2 b) { cfma(acc, a, b); }
-    __device__ __forceinline__ void join(int32_t off) {
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
-    }
-    __device__ __forceinline__ double2 value() const { return acc; }
-};
-
 // One pass of a tabulated small step: NP outputs per lane group, with table words t[], their shared
 // index split over the S = 2^lg lanes of the group.  The sums of the NP outputs are independent chains.
 template <typename T, int NP>

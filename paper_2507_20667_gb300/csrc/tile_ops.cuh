@@ -32,6 +32,59 @@ template <typename C> __device__ __forceinline__ C cscale(C v, decltype(C::x) s)
     return cmake(v.x * s, v.y * s);
 }
 
+// Error-free transformations (Knuth's TwoSum; the FMA form of Dekker's TwoProduct, as used by
+// Ogita, Rump and Oishi for accurate dot products), written with round-to-nearest intrinsics so
+// that the compiler neither contracts nor reorders them: a + b = s + err and a * b = p + err
+// exactly.
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &err) {
+    s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+// A sum kept as an unevaluated pair hi + lo (about 44 significant bits); adds x = xh + xl.
+__device__ __forceinline__ void df_add(float &hi, float &lo, float xh, float xl) {
+    float s, t;
+    two_sum(hi, xh, s, t);
+    hi = s;
+    lo = __fadd_rn(lo, __fadd_rn(xl, t));
+}
+
+// The sum of one output of a small step.  In complex64 Re and Im are kept as hi + lo pairs of exact
+// products and exact pairwise sums, rounded once when the output is stored: these steps are most of a
+// circuit's steps, and with plain FP32 multiply-adds their several roundings per output (rather than
+// the one of storing it) tripled the error of small amplitudes.
+template <typename T> struct SmallSum;
+template <> struct SmallSum<float> {
+    float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
+    __device__ __forceinline__ void mac(float2 a, float2 b) {
+        const float p1 = __fmul_rn(a.x, b.x), e1 = __fmaf_rn(a.x, b.x, -p1);
+        const float p2 = __fmul_rn(a.y, b.y), e2 = __fmaf_rn(a.y, b.y, -p2);
+        const float p3 = __fmul_rn(a.x, b.y), e3 = __fmaf_rn(a.x, b.y, -p3);
+        const float p4 = __fmul_rn(a.y, b.x), e4 = __fmaf_rn(a.y, b.x, -p4);
+        float s1, t1, s2, t2;
+        two_sum(p1, -p2, s1, t1);
+        two_sum(p3, p4, s2, t2);
+        df_add(rh, rl, s1, __fadd_rn(__fsub_rn(e1, e2), t1));
+        df_add(ih, il, s2, __fadd_rn(__fadd_rn(e3, e4), t2));
+    }
+    __device__ __forceinline__ void join(int32_t off) {
+        const float orh = __shfl_xor_sync(0xffffffffu, rh, off), orl = __shfl_xor_sync(0xffffffffu, rl, off);
+        const float oih = __shfl_xor_sync(0xffffffffu, ih, off), oil = __shfl_xor_sync(0xffffffffu, il, off);
+        df_add(rh, rl, orh, orl);
+        df_add(ih, il, oih, oil);
+    }
+    __device__ __forceinline__ float2 value() const { return cmake(__fadd_rn(rh, rl), __fadd_rn(ih, il)); }
+};
+template <> struct SmallSum<double> {
+    double2 acc = {0.0, 0.0};
+    __device__ __forceinline__ void mac(double2 a, double2 b) { cfma(acc, a, b); }
+    __device__ __forceinline__ void join(int32_t off) {
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
+    }
+    __device__ __forceinline__ double2 value() const { return acc; }
+};
+
 // frexp-style exponent of the float with bit pattern `bits` (0 for zero): x = f * 2^e with f in
 // [0.5, 1).  Subnormal maxima are treated as 2^-126.
 __device__ __forceinline__ int32_t scale_exponent(uint32_t bits) {
@@ -109,6 +162,14 @@ __device__ __forceinline__ void group_off2(const Groups &g, int64_t idx, int64_t
     }
 }
 
+// The same, out of line (for uses that are unrolled or rare).
+static __device__ __noinline__ int64_t group_off_call(const Groups *g, int64_t idx) { return group_off(*g, idx); }
+static __device__ __noinline__ longlong2 group_off2_call(const Groups *g, int64_t idx) {
+    int64_t a, b;
+    group_off2(*g, idx, a, b);
+    return make_longlong2(a, b);
+}
+
 // Copy a descriptor into shared memory (all threads), followed by a barrier.
 __device__ __forceinline__ void load_desc(StepDesc &dst, const StepDesc *src) {
     const int4 *s = reinterpret_cast<const int4 *>(src);
@@ -162,18 +223,18 @@ __device__ __forceinline__ void publish_max(float v, uint32_t *slot, float *red)
 }
 
 template <typename C>
-__device__ __forceinline__ const C *operand(const StepDesc &d, const JobPtrs &j, bool is_a) {
+__device__ __forceinline__ const C *operand(const StepHead &d, const JobPtrs &j, bool is_a) {
     const bool leaf = is_a ? (d.flags & FLAG_A_LEAF) : (d.flags & FLAG_B_LEAF);
     const int64_t off = is_a ? d.a_off : d.b_off;
     return leaf ? static_cast<const C *>(j.leaf) + off : reinterpret_cast<const C *>(j.arena) + off;
 }
 
-__device__ __forceinline__ void step_scales(const StepDesc &d, const JobPtrs &j, int32_t &eA, int32_t &eB) {
+__device__ __forceinline__ void step_scales(const StepHead &d, const JobPtrs &j, int32_t &eA, int32_t &eB) {
     eA = scale_exponent(__ldcg(j.maxbits + d.node_a));
     eB = scale_exponent(__ldcg(j.maxbits + d.node_b));
 }
 
-__device__ __forceinline__ void write_exponent(const StepDesc &d, const JobPtrs &j, int32_t eA, int32_t eB) {
+__device__ __forceinline__ void write_exponent(const StepHead &d, const JobPtrs &j, int32_t eA, int32_t eB) {
     j.exp2[d.node_c] = __ldcg(j.exp2 + d.node_a) + eA + __ldcg(j.exp2 + d.node_b) + eB;
 }
 
@@ -258,14 +319,47 @@ __device__ void tile_rows(const StepDesc &d, int64_t tile, const JobPtrs &j, cha
     if (tile == 0 && threadIdx.x == 0) write_exponent(d, j, eA, eB);
 }
 
-// Rotated shared-memory layout of a chained ROWS step's C (N a power of two): element (m, n) of
-// the dense row-major [M, N] tensor, dense index i = m N + n, sits at m N + ((n + (m >> r)) mod N)
-// with r = max(0, 4 - log2 N).  The threads of a warp each write their own row m; the rotation puts
-// their N-th outputs in 16 different 8-byte bank pairs.  The next step maps its dense A index
-// through the same function.
-__device__ __forceinline__ int32_t rot_index(int32_t i, int32_t lgn) {
-    const int32_t mask = (1 << lgn) - 1, r = lgn >= 4 ? 0 : 4 - lgn;
-    return (i & ~mask) | ((i + (i >> (lgn + r))) & mask);
+// A small step (the criterion of the subtree programs) that runs as a work tile of its own, complex64:
+// an output per thread, summed as the programs do (SmallSum), so that its value does not depend on
+// where it runs.
+__device__ __forceinline__ void tile_small(const StepDesc &d, const JobPtrs &j, char *smem, float *red) {
+    int2 *kt = reinterpret_cast<int2 *>(smem);   // [K <= 256] offsets in A and B
+    const int32_t N = (int32_t)d.N, K = (int32_t)d.K, O = (int32_t)d.M * N;
+    int32_t eA, eB;
+    step_scales(d, j, eA, eB);
+    const int32_t es = eA + eB;
+    const bool fold = es > -120 && es < 120;
+    const float sA = fold ? 1.f : pow2<float>(-eA), sB = fold ? pow2<float>(-es) : pow2<float>(-eB);
+    const float2 *__restrict__ A = operand<float2>(d, j, true);
+    const float2 *__restrict__ B = operand<float2>(d, j, false);
+    float2 *__restrict__ Cp = reinterpret_cast<float2 *>(j.arena) + d.c_off;
+    for (int32_t k = threadIdx.x; k < K; k += blockDim.x) {
+        const longlong2 o = group_off2_call(&d.k, k);
+        kt[k] = make_int2((int32_t)o.x, (int32_t)o.y);
+    }
+    __syncthreads();
+    float mx = 0.f;
+    for (int32_t o = threadIdx.x; o < O; o += blockDim.x) {
+        const float2 *a = A + group_off_call(&d.m, o / N), *b = B + group_off_call(&d.n, o % N);
+        SmallSum<float> sum;
+#pragma unroll 4
+        for (int32_t k = 0; k < K; ++k) sum.mac(cscale(ldc(a + kt[k].x), sA), cscale(ldc(b + kt[k].y), sB));
+        const float2 v = sum.value();
+        Cp[o] = v;
+        mx = fmaxf(mx, absmax2(v));
+    }
+    publish_max(mx, j.maxbits + d.node_c, red);
+    if (threadIdx.x == 0) write_exponent(d, j, eA, eB);
+}
+
+// Shared-memory layout of the large operand and of C of a staged step: element i of the dense row-major
+// tensor sits at swz(i) -- inside each run of 16 elements (128 bytes) its 16-byte pairs are exchanged
+// by an exclusive or with the higher index bits, so that threads that read or write elements 16 or more
+// apart spread over the banks.  Pairs stay pairs (16-byte copies work), and swz is linear over index
+// bits: swz(i | j) = swz(i) ^ swz(j) for disjoint bits.
+__host__ __device__ __forceinline__ uint32_t swz(uint32_t i) {
+    const uint32_t x = i >> 4;
+    return i ^ (((x ^ (x >> 3) ^ (x >> 6) ^ (x >> 9)) & 7u) << 1);
 }
 
 // Block-wide max of non-negative values, returned to every thread.  Ends with a barrier.
@@ -280,16 +374,6 @@ __device__ __forceinline__ float block_max(float v, float *red) {
     return v;
 }
 
-// ROWS step whose A fits in shared memory (complex64, FLAG_A_SMEM; the tile covers all M rows):
-// A is copied whole with 16-byte cp.async (coalesced) -- or, for a continuation of a chain
-// (A_ROT), is already in shared memory in the rotated layout of width 2^a_lgn -- and B densely and
-// scaled into the scratch area; each thread owns R = 32 / NT rows with their accumulators in
-// registers, reading A from shared memory (a row starts its shared index at m mod K when k is
-// contiguous in A, which keeps a warp's reads in different banks).  C then either stays in shared
-// memory in the rotated layout (c_in_smem: the next step of the chain consumes it; cmax receives
-// the block's max-abs of C) or is written into the same shared memory with padded rows and leaves
-// it in coalesced order.  HBM traffic: one read of A, one write of C, both coalesced (neither
-// for the inner steps of a chain).  Ends with a barrier.
 // Phase cycle accounting of the profiling variant of the dataflow kernel (PROF), compiled out of
 // the other one.
 template <bool PROF>
@@ -302,136 +386,264 @@ __device__ __forceinline__ void prof_phase(long long *prof, int slot, long long 
     }
 }
 
-template <int NT, bool A_ROT, bool PROF>
-__device__ void rows_smem_core(const StepDesc &d, const JobPtrs &j, char *smem, char *dyn, float *red,
-                               float sA, float sB, bool c_in_smem, float &cmax, long long *prof) {
+// cp.async of a staged step's A into its shared-memory layout (committed; the caller waits): swizzled for
+// power-of-two dims -- the index bits of rows and shared indices are then disjoint, and the address of an
+// entry is the exclusive or of its two parts -- else linear, where the parts add up.
+__device__ __forceinline__ void stage_a(const StepHead &d, const JobPtrs &j, float2 *As, int32_t MK, bool p2) {
+    const float2 *__restrict__ A = operand<float2>(d, j, true);
+#pragma unroll 2
+    for (int32_t i = threadIdx.x; 2 * i + 1 < MK; i += kThreads)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(As + (p2 ? swz(2 * i) : 2 * i))),
+                     "l"(A + 2 * i)
+                     : "memory");
+    if ((MK & 1) && threadIdx.x == 0)   // one entry, or no power of two
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(As + MK - 1)),
+                     "l"(A + MK - 1)
+                     : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// Step staged whole through shared memory (complex64, FLAG_A_SMEM; one tile covers the step): A is
+// copied with 16-byte cp.async into the swizzled layout -- or, for a continuation of a chain (a_res), is
+// there already, left by the previous step -- and B, scaled and dense, goes next to it.  Each thread owns
+// R rows x NC columns: the CG = rows_groups(N, NC) column groups lie on neighbouring lanes, the threads
+// of a group rstep rows apart.  C then stays in shared memory (c_in_smem: the next step of the chain
+// consumes it; the block's max-abs of C is returned) or leaves it in coalesced 16-byte stores.  Memory
+// traffic: one read of A and B, one write of C (B alone inside a chain).  Ends with a barrier.
+// Bound by shared-memory loads and the FMA pipe alike: a load instruction returns 128 bytes a cycle to the
+// registers of the SM whether or not its lanes share addresses, so a shared index costs a warp 2 R + 2 NC
+// cycles there against R NC of the pipe; 4 x 8 (24 against 32) keeps both short, where 2 x 16 took 36.
+// With the column groups on lanes, a load of A has 32 / CG different rows, which the swizzle spreads over
+// the banks, and one of B CG neighbouring pairs of columns.  Packed multiply-adds (fma.rn.f32x2) with B's
+// parts duplicated were slower: 16 bytes an entry.
+// Measured on 2432 24-qubit amplitudes (18 such steps in two chains each, 128 x 64 x 32, 256 x 32 x 32 and
+// 512 x 16 x 16 the largest): the dataflow kernel 2.05 ms; 2.99 ms with 2 x 16 thread tiles, N <= 16
+// only and the wider steps as separate GEMM tiles.
+// next: the step that continues the chain (null: none); its B is fetched while this step multiplies.
+// ahead: this step's B was fetched that way.
+constexpr int kAheadPer = kRowsAhead / kThreads;
+__device__ __forceinline__ int32_t b_entries(const StepHead &d) {
+    const int nc = rows_nc(d.tile_shape);
+    return (int32_t)d.K * rows_groups(d.N, nc) * nc;
+}
+__device__ __forceinline__ void b_ahead_offsets(const StepHead &d, const JobPtrs &j, int32_t (&o)[kAheadPer]) {
+    if (d.tile_shape == kRowsShapeSmall) return;
+    const int32_t *tab = reinterpret_cast<const int32_t *>(j.ktab + d.ktab_off) + d.M + d.K;
+    const int32_t n = b_entries(d);
+#pragma unroll
+    for (int q = 0; q < kAheadPer; ++q) {
+        const int32_t i = threadIdx.x + q * kThreads;
+        o[q] = i < n ? __ldg(tab + i) : -2;
+    }
+}
+__device__ __forceinline__ void b_ahead_copy(const StepHead &d, const JobPtrs &j, float2 *raw,
+                                             const int32_t (&o)[kAheadPer]) {
+    if (d.tile_shape == kRowsShapeSmall) return;
+    const float2 *B = operand<float2>(d, j, false);
+#pragma unroll
+    for (int q = 0; q < kAheadPer; ++q) {
+        const int32_t i = threadIdx.x + q * kThreads;
+        if (o[q] >= 0)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(raw + i)),
+                         "l"(B + o[q])
+                         : "memory");
+        else if (o[q] == -1) raw[i] = make_float2(0.f, 0.f);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+template <int NC, int R, bool PROF>
+__device__ float rows_smem_core(const StepHead &d, const JobPtrs &j, char *smem, char *dyn, float *red, int32_t eA,
+                                int32_t eB, bool a_res, bool ahead, const StepHead *next, long long *prof) {
     long long tp = 0;
     if (PROF && threadIdx.x == 0) tp = clock64();
     using C = float2;
-    constexpr int R = 32 / NT;
+    const int32_t M = (int32_t)d.M, N = (int32_t)d.N, K = (int32_t)d.K, MK = M * K;
+    const int32_t CG = rows_groups(N, NC), NB = CG * NC, rstep = kThreads / CG;
+    const int tid = threadIdx.x, cg = tid & (CG - 1);
+    // the step's table: byte offsets in A of its rows and of its shared indices, element offsets in B of
+    // its (k, column) entries (-1: no such column)
+    const int32_t *__restrict__ tab = reinterpret_cast<const int32_t *>(j.ktab + d.ktab_off);
+    int32_t *kat = reinterpret_cast<int32_t *>(smem);
     C *As = reinterpret_cast<C *>(dyn);
-    // [K][PB] scaled B, PB = N + 1 rounded up to even: rows start on 16 bytes and are read two
-    // entries per load
-    C *Bd = reinterpret_cast<C *>(smem);
-    int32_t *kat = reinterpret_cast<int32_t *>(Bd + 16 * (NT + 2));   // [K] offsets in A
-    const int32_t M = (int32_t)d.M, N = (int32_t)d.N, K = (int32_t)d.K, PB = (N + 2) & ~1, MK = M * K;
-    const int32_t PC = N + 1;   // padded C rows (M (N + 1) elements fit by construction)
-    const C *__restrict__ A = operand<C>(d, j, true);
+    char *Bp = smem + kRowsTabBytes;
+    if (K * NB * 8 > Scratch<float>::bytes - kRowsTabBytes) Bp = dyn + (MK * 8 + 15) / 16 * 16;
+    C *Bs = reinterpret_cast<C *>(Bp);
     const C *__restrict__ B = operand<C>(d, j, false);
-    C *__restrict__ Cp = reinterpret_cast<C *>(j.arena) + d.c_off;
-    const int tid = threadIdx.x;
-    if (!A_ROT) {
-        for (int32_t i = tid; 2 * i + 1 < MK; i += blockDim.x)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                             (uint32_t)__cvta_generic_to_shared(As + 2 * i)),
-                         "l"(A + 2 * i)
-                         : "memory");
-        if ((MK & 1) && tid == 0)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
-                             (uint32_t)__cvta_generic_to_shared(As + MK - 1)),
-                         "l"(A + MK - 1)
-                         : "memory");
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    }
-    for (int32_t i = tid; i < K * N; i += blockDim.x) {
-        const int32_t k = i / N, n = i - k * N;
-        int64_t oa, ob;
-        group_off2(d.k, k, oa, ob);
-        ob += group_off(d.n, n);
-        Bd[k * PB + n] = cscale(ldc(B + ob), sB);
-        if (n == 0) kat[k] = (int32_t)oa;
-    }
-    if (!A_ROT) asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();
-    prof_phase<PROF>(prof, 7, tp);
-    const int32_t lga = d.a_lgn;
-    const bool skew = d.k.n > 0 && d.k.sa[0] == 1;
-    const int32_t step = blockDim.x;
-    C acc[R][NT];
-    int32_t rows[R];
-    // rows m0 + r * step of this thread (one pass: M <= R * blockDim by construction)
-    const int32_t m0 = tid;
-    const int32_t sh = skew ? m0 % K : 0;
+    const bool p2 = (d.flags & FLAG_A_POW2) != 0, c_in_smem = next != nullptr;
+    if (!a_res) stage_a(d, j, As, MK, p2);
+    const int32_t m0 = tid / CG;
+    uint32_t row[R];   // absent rows read row 0
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int32_t m = m0 + r * step;
-        rows[r] = m < M ? (int32_t)group_off(d.m, m) : -1;
+    for (int r = 0; r < R; ++r) row[r] = m0 + r * rstep < M ? (uint32_t)__ldg(tab + m0 + r * rstep) : 0u;
+    if (tid < K) kat[tid] = __ldg(tab + M + tid);
+    int32_t onext[kAheadPer];   // where the next step's B entries are
+    if (c_in_smem) b_ahead_offsets(*next, j, onext);
+    // both scales on B where that keeps its entries normal numbers, else A's on A
+    const bool fold = eA > -60 && eA < 60 && eB > -60 && eB < 60;
+    const float sB = fold ? pow2<float>(-eA - eB) : pow2<float>(-eB);
+    C *raw = As + kRowsSmemElems;
+    if (!a_res) asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (ahead) {   // each thread reads what it copied itself
 #pragma unroll
-        for (int n = 0; n < NT; ++n) acc[r][n] = make_float2(0.f, 0.f);
-    }
-#pragma unroll 1
-    for (int32_t kk = 0; kk < K; ++kk) {
-        int32_t k = kk + sh;
-        if (k >= K) k -= K;
-        const int32_t ko = kat[k];
-        C av[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            int32_t ia = rows[r] + ko;
-            if (A_ROT) ia = rot_index(ia, lga);
-            av[r] = rows[r] >= 0 ? cscale(As[ia], sA) : make_float2(0.f, 0.f);
+        for (int q = 0; q < kAheadPer; ++q) {
+            const int32_t i = tid + q * kThreads;
+            if (i < K * NB) Bs[i] = cscale(raw[i], sB);
         }
-        const float4 *Bk = reinterpret_cast<const float4 *>(Bd + k * PB);
+    }
+#pragma unroll 4
+    for (int32_t i = tid + (ahead ? kRowsAhead : 0); i < K * NB; i += kThreads) {
+        const int32_t o = __ldg(tab + M + K + i);
+        Bs[i] = o >= 0 ? cscale(ldc(B + o), sB) : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    if (c_in_smem) b_ahead_copy(*next, j, raw, onext);
+    if (!fold) {
+        const float sA = pow2<float>(-eA);
+#pragma unroll 1
+        for (int32_t i = tid; i < (MK + 15) / 16 * 16; i += kThreads) As[i] = cscale(As[i], sA);
+        __syncthreads();
+    }
+    prof_phase<PROF>(prof, 7, tp);
+    C acc[R][NC];
 #pragma unroll
-        for (int n2 = 0; n2 < NT / 2; ++n2) {
-            if (2 * n2 >= N) break;
-            const float4 bb = Bk[n2];
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int n = 0; n < NC; ++n) acc[r][n] = make_float2(0.f, 0.f);
+    const C *Bk = Bs + 2 * cg;   // column n of the thread: (n / 2) 2 CG + 2 cg + n mod 2
+    const uint32_t carry = p2 ? 0u : ~0u;   // x + y = (x ^ y) + 2 (x & y)
+#pragma unroll 2
+    for (int32_t k = 0; k < K; ++k, Bk += NB) {
+        const uint32_t ko = (uint32_t)kat[k];
+        C a[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            a[r] = *reinterpret_cast<const C *>(reinterpret_cast<const char *>(As) + (row[r] ^ ko) +
+                                                (2 * (row[r] & ko) & carry));
+#pragma unroll
+        for (int n = 0; n < NC; n += 2) {
+            const float4 bb = *reinterpret_cast<const float4 *>(Bk + n * CG);
             const C b0 = make_float2(bb.x, bb.y), b1 = make_float2(bb.z, bb.w);
 #pragma unroll
-            for (int r = 0; r < R; ++r) cfma(acc[r][2 * n2], av[r], b0);
-            if (2 * n2 + 1 < N) {
+            for (int r = 0; r < R; ++r) cfma(acc[r][n], a[r], b0);
 #pragma unroll
-                for (int r = 0; r < R; ++r) cfma(acc[r][2 * n2 + 1], av[r], b1);
+            for (int r = 0; r < R; ++r) cfma(acc[r][n + 1], a[r], b1);
+        }
+    }
+    __syncthreads();   // every thread is done reading A and B
+    prof_phase<PROF>(prof, 11, tp);
+    float mx = 0.f;
+    // columns past N are sums of zeros
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int n = 0; n < NC; ++n) mx = fmaxf(mx, absmax2(acc[r][n]));
+    if (NB == N) {   // a power of two: row and column bits are disjoint, and a pair is one 16-byte piece
+        uint32_t cs[NC / 2];
+#pragma unroll
+        for (int n = 0; n < NC / 2; ++n) cs[n] = swz((uint32_t)(2 * n * CG + 2 * cg));
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int32_t m = m0 + r * rstep;
+            const uint32_t mrow = swz((uint32_t)(m * N));
+            if (m < M) {
+#pragma unroll
+                for (int n = 0; n < NC / 2; ++n)
+                    *reinterpret_cast<float4 *>(As + (mrow ^ cs[n])) =
+                        make_float4(acc[r][2 * n].x, acc[r][2 * n].y, acc[r][2 * n + 1].x, acc[r][2 * n + 1].y);
             }
         }
+    } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int32_t m = m0 + r * rstep;
+#pragma unroll
+            for (int n = 0; n < NC; ++n) {
+                const int32_t c = (n / 2) * 2 * CG + 2 * cg + (n & 1);
+                if (m < M && c < N) As[swz((uint32_t)(m * N + c))] = acc[r][n];
+            }
+        }
+    }
+    if (c_in_smem) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");   // the next step's B and the head after it
+        const float cmax = block_max(mx, red);
+        prof_phase<PROF>(prof, 15, tp);
+        return cmax;
+    }
+    __syncthreads();
+    C *__restrict__ Cp = reinterpret_cast<C *>(j.arena) + d.c_off;   // 256-byte aligned
+    const int32_t MN = M * N;
+    for (int32_t i = 2 * tid; i + 1 < MN; i += 2 * kThreads)
+        *reinterpret_cast<float4 *>(Cp + i) = *reinterpret_cast<const float4 *>(As + swz((uint32_t)i));
+    if ((MN & 1) && tid == 0) Cp[MN - 1] = As[swz((uint32_t)(MN - 1))];
+    publish_max(mx, j.maxbits + d.node_c, red);
+    prof_phase<PROF>(prof, 15, tp);
+    return 0.f;
+}
+
+// A small step (the criterion of the subtree programs: at most 256 outputs) staged the same way, an
+// output per thread, summed as the programs do.  Its table: A offsets of rows and shared indices as
+// above, then element offsets in B of the shared indices and of the columns.
+template <bool PROF>
+__device__ float rows_smem_small(const StepHead &d, const JobPtrs &j, char *dyn, float *red, int32_t eA, int32_t eB,
+                                 bool a_res, const StepHead *next, long long *prof) {
+    long long tp = 0;
+    if (PROF && threadIdx.x == 0) tp = clock64();
+    using C = float2;
+    const int32_t M = (int32_t)d.M, N = (int32_t)d.N, K = (int32_t)d.K, o = threadIdx.x;
+    const int32_t *__restrict__ tab = reinterpret_cast<const int32_t *>(j.ktab + d.ktab_off);
+    C *As = reinterpret_cast<C *>(dyn);
+    const bool p2 = (d.flags & FLAG_A_POW2) != 0, c_in_smem = next != nullptr, act = o < M * N;
+    if (!a_res) {
+        stage_a(d, j, As, M * K, p2);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+    }
+    if (c_in_smem) {
+        int32_t onext[kAheadPer];
+        b_ahead_offsets(*next, j, onext);
+        b_ahead_copy(*next, j, As + kRowsSmemElems, onext);
+    }
+    const int32_t es = eA + eB;
+    const bool fold = es > -120 && es < 120;
+    const float sA = fold ? 1.f : pow2<float>(-eA), sB = fold ? pow2<float>(-es) : pow2<float>(-eB);
+    const uint32_t row = act ? (uint32_t)__ldg(tab + o / N) : 0u, carry = p2 ? 0u : ~0u;
+    const C *B = operand<C>(d, j, false) + (act ? __ldg(tab + M + 2 * K + o % N) : 0);
+    SmallSum<float> sum;
+#pragma unroll 4
+    for (int32_t k = 0; k < K; ++k) {
+        const uint32_t ko = (uint32_t)__ldg(tab + M + k);
+        const C a = *reinterpret_cast<const C *>(reinterpret_cast<const char *>(As) + (row ^ ko) +
+                                                 (2 * (row & ko) & carry));
+        sum.mac(cscale(a, sA), cscale(ldc(B + __ldg(tab + M + K + k)), sB));
     }
     __syncthreads();   // every thread is done reading A
     prof_phase<PROF>(prof, 11, tp);
-    float mx = 0.f;
+    const C v = sum.value();
     if (c_in_smem) {
-        const int32_t lgn = __ffs(N) - 1, rs = lgn >= 4 ? 0 : 4 - lgn;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int32_t m = m0 + r * step;
-            if (m >= M) continue;
-#pragma unroll
-            for (int n = 0; n < NT; ++n)
-                if (n < N) {
-                    As[m * N + ((n + (m >> rs)) & (N - 1))] = acc[r][n];
-                    mx = fmaxf(mx, absmax2(acc[r][n]));
-                }
-        }
-        cmax = block_max(mx, red);
-        prof_phase<PROF>(prof, 15, tp);
-        return;
+        if (act) As[swz((uint32_t)o)] = v;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        return block_max(act ? absmax2(v) : 0.f, red);
     }
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int32_t m = m0 + r * step;
-        if (m >= M) continue;
-#pragma unroll
-        for (int n = 0; n < NT; ++n)
-            if (n < N) {
-                As[m * PC + n] = acc[r][n];
-                mx = fmaxf(mx, absmax2(acc[r][n]));
-            }
-    }
-    __syncthreads();
-    for (int32_t i = tid; i < M * N; i += blockDim.x) {
-        const int32_t m = i / N;
-        Cp[i] = As[m * PC + (i - m * N)];
-    }
-    publish_max(mx, j.maxbits + d.node_c, red);
-    prof_phase<PROF>(prof, 15, tp);
+    if (act) (reinterpret_cast<C *>(j.arena) + d.c_off)[o] = v;
+    publish_max(act ? absmax2(v) : 0.f, j.maxbits + d.node_c, red);
+    return 0.f;
 }
 
-template <bool A_ROT, bool PROF>
-__device__ __forceinline__ void rows_smem_any(const StepDesc &d, const JobPtrs &j, char *smem, char *dyn,
-                                              float *red, float sA, float sB, bool c_in_smem, float &cmax,
-                                              long long *prof) {
-    if (d.N <= 4) rows_smem_core<4, A_ROT, PROF>(d, j, smem, dyn, red, sA, sB, c_in_smem, cmax, prof);
-    else if (d.N <= 8) rows_smem_core<8, A_ROT, PROF>(d, j, smem, dyn, red, sA, sB, c_in_smem, cmax, prof);
-    else rows_smem_core<16, A_ROT, PROF>(d, j, smem, dyn, red, sA, sB, c_in_smem, cmax, prof);
+// The thread tile of a staged step: the smallest that covers it (see rows_shape).
+template <bool PROF>
+__device__ __forceinline__ float rows_smem_any(const StepHead &d, const JobPtrs &j, char *smem, char *dyn, float *red,
+                                               int32_t eA, int32_t eB, bool a_res, bool ahead, const StepHead *next,
+                                               long long *prof) {
+    switch (d.tile_shape) {
+        case 0: return rows_smem_core<rows_nc(0), rows_r(0), PROF>(d, j, smem, dyn, red, eA, eB, a_res, ahead, next, prof);
+        case 1: return rows_smem_core<rows_nc(1), rows_r(1), PROF>(d, j, smem, dyn, red, eA, eB, a_res, ahead, next, prof);
+        case 2: return rows_smem_core<rows_nc(2), rows_r(2), PROF>(d, j, smem, dyn, red, eA, eB, a_res, ahead, next, prof);
+        case 3: return rows_smem_core<rows_nc(3), rows_r(3), PROF>(d, j, smem, dyn, red, eA, eB, a_res, ahead, next, prof);
+        default: return rows_smem_small<PROF>(d, j, dyn, red, eA, eB, a_res, next, prof);
+    }
 }
 
 // A ROWS step staged through shared memory on its own.
@@ -439,47 +651,66 @@ __device__ __forceinline__ void tile_rows_smem(const StepDesc &d, const JobPtrs 
                                                float *red) {
     int32_t eA, eB;
     step_scales(d, j, eA, eB);
-    float cmax = 0.f;
-    rows_smem_any<false, false>(d, j, smem, dyn, red, pow2<float>(-eA), pow2<float>(-eB), false, cmax, nullptr);
+    rows_smem_any<false>(d, j, smem, dyn, red, eA, eB, false, false, nullptr, nullptr);
     if (threadIdx.x == 0) write_exponent(d, j, eA, eB);
 }
 
-// A chain of ROWS steps linked by chain_next, run by one block of the persistent kernel: the first
+// A chain of staged steps linked by chain_next, run by one block of the persistent kernel: the first
 // step reads A from the arena, each later one takes the previous step's C, kept in shared memory,
 // as its A, and the last writes its C to the arena.  The per-step power-of-two scaling is
 // unchanged: a continuation's A exponent comes from the block max of the previous C, which is the
 // value the separate steps would publish, so results are bit-identical to running the steps one
 // by one; the exponents of the inner nodes stay in registers and only the last node's max-abs and
-// exponent are written.  d is the block's shared descriptor and is overwritten with each step's;
-// thread 0 writes the indices of the continuation steps to chain[].  Returns their count.
+// exponent are written.  The heads of the steps are fetched two steps ahead into a ring of three, and
+// the next step's B and its scale one step ahead, so that inside a chain no step waits for them.
+// Thread 0 writes the indices of the continuation steps to chain[].  Returns their count.
+constexpr int kHeadPieces = (int)(sizeof(StepHead) / 16);
+__device__ __forceinline__ void head_copy(StepHead &dst, const StepDesc *src) {   // asynchronous, not committed
+    if (threadIdx.x < kHeadPieces)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(reinterpret_cast<char *>(&dst) + 16 * threadIdx.x)),
+                     "l"(reinterpret_cast<const char *>(static_cast<const StepHead *>(src)) + 16 * threadIdx.x)
+                     : "memory");
+}
+
 template <bool PROF>
-__device__ __forceinline__ int32_t rows_chain(StepDesc &d, const JobPtrs &j, char *smem, char *dyn, float *red,
-                                              int32_t *chain, long long *prof) {
+__device__ __forceinline__ int32_t rows_chain(const StepDesc &d, const JobPtrs &j, char *smem, char *dyn, float *red,
+                                              StepHead *ring, int32_t *chain, long long *prof) {
+    head_copy(ring[1], j.steps + d.chain_next);
+    asm volatile("cp.async.commit_group;" ::: "memory");
     int32_t eA, eB;
     step_scales(d, j, eA, eB);
     int32_t xa = __ldcg(j.exp2 + d.node_a), xb = __ldcg(j.exp2 + d.node_b);
-    int32_t n = 0;
+    if (threadIdx.x < kHeadPieces)
+        reinterpret_cast<int4 *>(ring)[threadIdx.x] = reinterpret_cast<const int4 *>(&d)[threadIdx.x];
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    int32_t n = 0, at = 0;   // step of the chain, its place in the ring
     while (true) {
-        const int32_t next = d.chain_next;
-        int4 dr[kDescRounds];
-        if (next >= 0) desc_fetch(dr, j.steps + next);
-        float cmax = 0.f;
-        const float sA = pow2<float>(-eA), sB = pow2<float>(-eB);
-        if (n == 0) rows_smem_any<false, PROF>(d, j, smem, dyn, red, sA, sB, next >= 0, cmax, prof);
-        else rows_smem_any<true, PROF>(d, j, smem, dyn, red, sA, sB, next >= 0, cmax, prof);
+        const StepHead &cur = ring[at];
+        const int32_t after = at == 2 ? 0 : at + 1;
+        const StepHead *next = cur.chain_next >= 0 ? ring + after : nullptr;
+        uint32_t next_max = 0;
+        int32_t next_exp = 0;
+        if (next) {
+            if (next->chain_next >= 0) head_copy(ring[after == 2 ? 0 : after + 1], j.steps + next->chain_next);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            next_max = __ldcg(j.maxbits + next->node_b);
+            next_exp = __ldcg(j.exp2 + next->node_b);
+        }
+        const float cmax = rows_smem_any<PROF>(cur, j, smem, dyn, red, eA, eB, n > 0, n > 0, next, prof);
         const int32_t xc = xa + eA + xb + eB;
-        if (next < 0) {
-            if (threadIdx.x == 0) j.exp2[d.node_c] = xc;
+        if (!next) {
+            if (threadIdx.x == 0) j.exp2[cur.node_c] = xc;
             return n;
         }
-        desc_store(dr, d);   // the step ended with a barrier: nobody reads the old descriptor
-        __syncthreads();
-        if (threadIdx.x == 0) chain[n] = next;
+        if (threadIdx.x == 0) chain[n] = cur.chain_next;
         ++n;
+        at = after;
         xa = xc;
         eA = scale_exponent(__float_as_uint(cmax));
-        eB = scale_exponent(__ldcg(j.maxbits + d.node_b));
-        xb = __ldcg(j.exp2 + d.node_b);
+        eB = scale_exponent(next_max);
+        xb = next_exp;
     }
 }
 
@@ -487,6 +718,10 @@ template <typename T>
 __device__ __forceinline__ void tile_rows_dispatch(const StepDesc &d, int64_t tile, const JobPtrs &j,
                                                    char *smem, float *red, char *dyn) {
     if constexpr (sizeof(T) == 4) {
+        if (d.flags & FLAG_SMALL) {
+            tile_small(d, j, smem, red);
+            return;
+        }
         if (d.flags & FLAG_A_SMEM) {
             tile_rows_smem(d, j, smem, dyn, red);
             return;

@@ -423,3 +423,43 @@ def test_long_dots(tnsa, dims, shift, transposed, precision):
     # most on the way of a term); complex128: 8 products and then a sum per burst
     eps = 16 * 2.0 ** -24 if precision == "c64" else (64 + math.prod(dims) / 2048) * 2.0 ** -53
     assert abs(m * 2.0 ** e - ref) <= 2 * eps * scale
+
+
+# steps staged whole through shared memory, alone and as a chain of two: every thread tile, its largest row
+# counts, widths and shared indices that are no powers of two, entries past one fetch ahead, and sizes past
+# the limits (which run as other steps); factors near the ends of the FP32 range move the scales to A
+@pytest.mark.parametrize("shape", [(512, 16, 16), (1024, 8, 8), (2048, 4, 4), (256, 32, 32), (128, 64, 32), (144, 64, 64),
+                                   (512, 2, 4), (2048, 1, 4), (300, 5, 7), (100, 20, 33), (511, 17, 3), (2047, 3, 2),
+                                   (9, 63, 64), (129, 64, 32), (513, 16, 16), (140, 60, 65), (2, 40, 50)])
+@pytest.mark.parametrize("tail", [0, 8])
+@pytest.mark.parametrize("magnitude", [1.0, 2.0 ** 100])
+def test_staged_step_shapes(tnsa, shape, tail, magnitude):
+    M, N, K = shape
+    rng = np.random.default_rng(M * 64 + N)
+
+    def normal(*s):
+        return rng.standard_normal(s) + 1j * rng.standard_normal(s)
+    x, y, b = normal(M, 2) * magnitude, normal(2, K), normal(K, N) / magnitude
+    f, d = (normal(N, tail), normal(M, tail)) if tail else (None, normal(M, N))
+    tensors = [x, y, b] + ([f] if tail else []) + [d]
+    last = len(tensors) - 1
+    edges = [(0, 1, 1, 0), (1, 1, 2, 0), (0, 0, last, 0)]
+    edges += [(2, 1, 3, 0), (3, 1, 4, 1)] if tail else [(2, 1, 3, 1)]
+    net = tni.Network(tensors, np.array(edges, np.int32), np.zeros(len(tensors), np.int32), ["t"] * len(tensors))
+    h = tnsa.tn_build(net)
+    n = len(tensors)
+    plan = tnsa.tn_plan_import(h, [(0, 1)] + [(n + i, 2 + i) for i in range(n - 2)])
+    c = tnsa.tn_ctx_create(0)
+    out = []
+    for chains in (1, 0):
+        tnsa.tn_ctx_set_config(c, local_budget=0, rows_chains=chains)
+        m, e, _ = tnsa.tn_contract(c, h, plan, "c64")
+        out.append(m * 2.0 ** e)
+    assert out[0] == out[1]
+
+    def value(*t):
+        r = t[0] @ t[1] @ t[2]
+        return ((r @ t[3] if tail else r) * t[-1]).sum()
+    # one rounding per leaf and stored step, two per term of a sum of K (or N, 2) complex products, 16 in the dot
+    eps = (2 * (K + 2 + (N if tail else 0)) + 24) * 2.0 ** -24
+    assert abs(out[0] - value(*tensors)) <= eps * value(*(np.abs(t) for t in tensors))
