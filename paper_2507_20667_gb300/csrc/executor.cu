@@ -283,10 +283,13 @@ size_t plan_memory(const Plan &plan, int32_t n, const std::vector<size_t> &bytes
 }
 
 // Rows per work tile of a global ROWS step: large enough to amortise the tile's fixed cost
-// (descriptor, scales, B staging, completion fence), 16 rows per thread at most.
-int32_t rows_per_tile(int64_t M) {
-    if (M <= 4096) return (int32_t)std::max<int64_t>(M, 1);
-    return 4096;
+// (descriptor, scales, B staging, completion fence), 16 rows per thread at most.  Complex128 tiles hold
+// about 8192 multiply-adds instead: at the FP64 rate these take 16 k cycles, twice the fixed cost, and a
+// 4096 x 16 x 4 step in one tile held up its job for 140 k cycles while other SMs idled.
+int32_t rows_per_tile(int64_t M, int64_t N, int64_t K, int32_t elem) {
+    int64_t rows = 4096;
+    if (elem == 16) rows = std::min(rows, std::max<int64_t>(kThreads, 8192 / (N * K) / kThreads * kThreads));
+    return (int32_t)std::max<int64_t>(1, std::min(M, rows));
 }
 
 // The thread tile of a step staged whole through shared memory: the smallest one whose threads cover M
@@ -933,7 +936,7 @@ tn_status tn::compile(Compiled &c, const Net &net, const Plan &plan, const Compi
             c.counts[STEP_ROWS]++;
         } else if (N <= kRowsMaxN && K <= kRowsMaxK && K * N <= kRowsMaxKN) {
             d.kind = STEP_ROWS;
-            d.tile_rows = rows_per_tile(M);
+            d.tile_rows = rows_per_tile(M, N, K, elem);
             d.ntiles = (int32_t)((M + d.tile_rows - 1) / d.tile_rows);
             c.steps.push_back(d);
             c.counts[STEP_ROWS]++;
@@ -955,10 +958,14 @@ tn_status tn::compile(Compiled &c, const Net &net, const Plan &plan, const Compi
             c.counts[STEP_TC]++;
         } else {
             d.kind = STEP_TILE;
-            // narrow complex64 outputs (N <= 32) use 128 x 32 tiles so no thread computes padding
-            const bool narrow = N <= kTileN / 2 && elem == 8;
-            d.tile_rows = narrow ? kTileNarrow : 0;
-            const int64_t tm = narrow ? 2 * kTileM : kTileM, tn = narrow ? kTileN / 2 : kTileN;
+            // complex64: few outputs and a long shared index split the latter over thread groups, narrow
+            // outputs (N <= 32) leave no thread to compute padding; complex128, bound by FP64 (a tile's
+            // 32 x 32 x 16 takes 33 k cycles), uses small tiles so that a small batch fills the SMs
+            d.tile_rows = elem != 8                        ? TILE_C128
+                          : M * N <= 4096 && K >= 256      ? TILE_LONG_K
+                          : N <= tile_n(TILE_NARROW)       ? TILE_NARROW
+                                                           : TILE_SQUARE;
+            const int64_t tm = tile_m(d.tile_rows), tn = tile_n(d.tile_rows);
             const int64_t tiles = ((M + tm - 1) / tm) * ((N + tn - 1) / tn);
             if (tiles > 0x7fffffffLL) return fail(TN_EUNSUPPORTED, "step too large");
             d.ntiles = (int32_t)tiles;

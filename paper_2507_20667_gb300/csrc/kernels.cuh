@@ -62,7 +62,7 @@ struct StepHead {
     int32_t ntiles;                // work tiles of this step
     int32_t dep0, dep1;            // steps producing A and B (-1: a leaf); DOTF: dep0 = its DOTP
     int32_t tile_rows;             // ROWS: output rows per tile; DOTP: shared indices per tile;
-                                   // TILE: tile shape (0: 64 x 64, kTileNarrow: 128 x 32)
+                                   // TILE: TileShape
     int32_t part_off;              // DOTP / DOTF: offset of the step's partials (in double2)
     int32_t level;                 // longest path from the leaves (scheduling order)
     int32_t ktab_off;              // DOTP: first entry of its shared-index offset table (-1: none);
@@ -251,8 +251,10 @@ cudaError_t launch_permute(const void *src, void *dst, int32_t elem_bytes, int32
 
 // Tiling constants shared by the compiler and the kernels.
 constexpr int kThreads = 256;
-constexpr int kTileM = 64, kTileN = 64, kTileK = 16;   // CUDA-core GEMM tile
-constexpr int kTileNarrow = 1;                          // TILE: tile_rows = 1 selects 128 x 32 tiles
+// CUDA-core GEMM tiles (StepDesc.tile_rows of a TILE step): output rows and columns.
+enum TileShape : int32_t { TILE_SQUARE = 0, TILE_NARROW = 1, TILE_LONG_K = 2, TILE_C128 = 3 };
+constexpr int tile_m(int shape) { return shape == TILE_SQUARE ? 64 : shape == TILE_NARROW ? 128 : shape == TILE_LONG_K ? 16 : 32; }
+constexpr int tile_n(int shape) { return shape == TILE_SQUARE ? 64 : shape == TILE_LONG_K ? 16 : 32; }
 constexpr int kRowsMaxKN = 1024, kRowsMaxK = 64, kRowsMaxN = 16;
 constexpr int kDotMaxOut = 4;
 // Steps staged whole through shared memory (complex64): A (M K elements), B where it does not fit the

@@ -243,9 +243,10 @@ template <typename T> struct Scratch {
     using C = cx_t<T>;
     static constexpr int TK_MM = sizeof(T) == 4 ? 8 : 4;   // shared-index chunk of local_mm
     static constexpr int rows = kRowsMaxKN * sizeof(C) + kRowsMaxK * sizeof(int64_t);
-    // GEMM operand tiles and index arrays: 64 x 64, and for complex64 also 128 x 32 (the larger)
-    static constexpr int tile_cols = sizeof(T) == 4 ? 2 * kTileM + kTileN / 2 : kTileM + kTileN;
-    static constexpr int tile = kTileK * tile_cols * sizeof(C) + (tile_cols + 4 * kTileK) * sizeof(int64_t);
+    // GEMM: two stages of operand tiles, the largest 8 shared indices of 128 + 32 rows (complex64), of 32 + 32
+    // (complex128), and the index arrays
+    static constexpr int tile_rows = sizeof(T) == 4 ? 160 : 64;
+    static constexpr int tile = 2 * 8 * (tile_rows + 2) * (int)sizeof(C) + (tile_rows + 48) * (int)sizeof(int64_t);
     static constexpr int dot = (kThreads / 32) * kDotMaxOut * sizeof(double2) + 2 * kDotMaxOut * sizeof(int64_t);
     // subtree programs: the register-tiled GEMM's operand tiles and offsets, or the REDUCE mode's
     // offset table and FP64 partials
@@ -735,109 +736,172 @@ __device__ __forceinline__ void tile_rows_dispatch(const StepDesc &d, int64_t ti
 }
 
 // ------------------------------------------------------------------------------ TILE (GEMM)
-// General contraction on CUDA cores: a TM x TN output tile (64 x 64, or 128 x 32 for narrow N),
-// K in chunks of kTileK, operand tiles gathered through the index maps into shared memory, 4 x 4
-// outputs per thread.  The gathers of chunk c + 1 are issued into registers before chunk c is
-// computed, so their latency overlaps the arithmetic.
-template <typename T, int TM, int TN>
+// General contraction on CUDA cores: a TM x TN output tile, RM x RN outputs per thread, the shared index
+// in chunks of KS TK: the block's KS thread groups take TK shared indices of a chunk each (their sums are
+// added in a fixed order at the end).  Operand chunks are gathered through the index maps into shared
+// memory with cp.async, chunk c + 1 while chunk c is multiplied, running along whichever index is
+// contiguous in the operand, so that a warp reads whole sectors.  Both scales are applied to the sums;
+// where they are too large for that (the products of unscaled entries could leave FP32's range) to the
+// gathered entries.
+// Bound by the FMA pipe (56 % of it at two blocks per SM) and by the last wave of tiles, which run alone
+// on their SMs: 128 x 64 tiles with 8 x 4 outputs a thread spent as much per multiply-add and had the
+// longer tail.  Measured, a 64 x 64 x 512 complex64 tile: 236 k cycles, 308 k with register-staged gathers
+// along the rows.  Few outputs with a long shared index take KS = 4: 8 x 8 x 512 took 250 k cycles in a
+// 64 x 64 tile and takes 45 k.
+template <typename T, int TM, int TN, int RM, int RN, int TK, int KS>
 __device__ void tile_gemm(const StepDesc &d, int64_t tile, const JobPtrs &j, char *smem, float *red) {
     using C = cx_t<T>;
-    constexpr int TX = TN / 4, TY = TM / 4;
-    static_assert(TX * TY == kThreads, "one 4 x 4 register tile per thread");
-    constexpr int RA = TM * kTileK / kThreads, RB = TN * kTileK / kThreads;
-    static_assert(RA * kThreads == TM * kTileK && RB * kThreads == TN * kTileK, "operand tile split");
-    C(*As)[TM] = reinterpret_cast<C(*)[TM]>(smem);
-    C(*Bs)[TN] = reinterpret_cast<C(*)[TN]>(smem + kTileK * TM * sizeof(C));
-    int64_t *rowA = reinterpret_cast<int64_t *>(smem + kTileK * (TM + TN) * sizeof(C));
+    constexpr int TX = TN / RN, TY = TM / RM, KC = TK * KS, PA = TM + 1, PB = TN + 1;
+    static_assert(TX * TY * KS == kThreads, "one register tile per thread");
+    constexpr int RA = TM * KC / kThreads, RB = TN * KC / kThreads;
+    static_assert(RA * kThreads == TM * KC && RB * kThreads == TN * KC, "operand tile split");
+    static_assert((KS & (KS - 1)) == 0 && KC <= kThreads, "thread groups");
+    constexpr int stage = KC * (PA + PB), tile_bytes = (2 * stage * (int)sizeof(C) + 7) / 8 * 8;
+    static_assert(tile_bytes + (TM + TN + 6 * KC) * 8 <= Scratch<T>::bytes, "scratch");
+    static_assert(KS / 2 * TM * TN * (int)sizeof(C) <= Scratch<T>::bytes, "partial sums");
+    C *As = reinterpret_cast<C *>(smem);   // [2 stages][KC][PA], then [KC][PB] of the same stage
+    int64_t *rowA = reinterpret_cast<int64_t *>(smem + tile_bytes);
     int64_t *colB = rowA + TM;
-    int64_t(*kAo)[kTileK] = reinterpret_cast<int64_t(*)[kTileK]>(colB + TN);   // [2][kTileK]
-    int64_t(*kBo)[kTileK] = kAo + 2;
+    int64_t *kAo = colB + TN, *kBo = kAo + 3 * KC;   // [3][KC], written two chunks ahead
     const int64_t M = d.M, N = d.N, K = d.K;
     const int64_t tiles_n = (N + TN - 1) / TN;
     const int64_t m0 = (tile / tiles_n) * TM, n0 = (tile % tiles_n) * TN;
     int32_t eA, eB;
     step_scales(d, j, eA, eB);
-    const T sA = pow2<T>(-eA), sB = pow2<T>(-eB);
+    constexpr int kLate = sizeof(T) == 4 ? 40 : 120;   // |exponents| up to which the sums are scaled
+    const bool late = eA > -kLate && eA < kLate && eB > -kLate && eB < kLate;
     const C *__restrict__ A = operand<C>(d, j, true);
     const C *__restrict__ B = operand<C>(d, j, false);
     C *__restrict__ Cp = reinterpret_cast<C *>(j.arena) + d.c_off;
     const int tid = threadIdx.x;
+    const bool a_k = d.k.n > 0 && d.k.sa[0] == 1, b_k = d.k.n > 0 && d.k.sb[0] == 1;   // contiguous along k
     for (int i = tid; i < TM + TN; i += kThreads) {
         if (i < TM) rowA[i] = (m0 + i < M) ? group_off(d.m, m0 + i) : -1;
         else colB[i - TM] = (n0 + i - TM < N) ? group_off(d.n, n0 + i - TM) : -1;
     }
-    const int64_t nch = (K + kTileK - 1) / kTileK;
-    auto koffs = [&](int64_t c) {
-        if (tid < kTileK) {
-            const int64_t k = c * kTileK + tid;
+    const int32_t nch = (int32_t)((K + KC - 1) / KC);
+    auto koffs = [&](int32_t c, int slot) {
+        if (tid < KC) {
+            const int64_t k = (int64_t)c * KC + tid;
             int64_t oa = -1, ob = -1;
-            if (k < K) group_off2(d.k, k, oa, ob);
-            kAo[c & 1][tid] = oa;
-            kBo[c & 1][tid] = ob;
+            if (k < K) {
+                if (d.k.n == 1) {
+                    oa = k * d.k.sa[0];
+                    ob = k * d.k.sb[0];
+                } else {
+                    group_off2(d.k, k, oa, ob);
+                }
+            }
+            kAo[slot * KC + tid] = oa;
+            kBo[slot * KC + tid] = ob;
         }
     };
-    C ra[RA], rb[RB];
-    auto gather = [&](int64_t c) {
-        const int64_t *ka = kAo[c & 1], *kb = kBo[c & 1];
+    auto copy = [&](C *dst, const C *src, bool in) {
+        if (!in) *dst = cmake((T)0, (T)0);
+        else
+            asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                         "l"(src), "n"(sizeof(C))
+                         : "memory");
+    };
+    auto gather = [&](int st, int slot) {
+        C *a = As + st * stage, *b = a + KC * PA;
+        const int64_t *ka = kAo + slot * KC, *kb = kBo + slot * KC;
 #pragma unroll
         for (int r = 0; r < RA; ++r) {
-            const int i = tid + r * kThreads, row = i % TM, kk = i / TM;
-            ra[r] = (rowA[row] >= 0 && ka[kk] >= 0) ? ldc(A + rowA[row] + ka[kk]) : cmake((T)0, (T)0);
+            const int i = tid + r * kThreads, row = a_k ? i / KC : i % TM, kk = a_k ? i % KC : i / TM;
+            const int64_t o = rowA[row], ok = ka[kk];
+            copy(a + kk * PA + row, A + o + ok, (o | ok) >= 0);
         }
 #pragma unroll
         for (int r = 0; r < RB; ++r) {
-            const int i = tid + r * kThreads, col = i % TN, kk = i / TN;
-            rb[r] = (colB[col] >= 0 && kb[kk] >= 0) ? ldc(B + kb[kk] + colB[col]) : cmake((T)0, (T)0);
+            const int i = tid + r * kThreads, col = b_k ? i / KC : i % TN, kk = b_k ? i % KC : i / TN;
+            const int64_t o = colB[col], ok = kb[kk];
+            copy(b + kk * PB + col, B + o + ok, (o | ok) >= 0);
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    koffs(0);
+    koffs(0, 0);
+    koffs(1, 1);
     __syncthreads();
-    gather(0);
-    const int tx = tid % TX, ty = tid / TX;
-    C acc[4][4];
+    gather(0, 0);
+    const int tx = tid % TX, ty = tid / TX % TY, ks = tid / (TX * TY);
+    C acc[RM][RN];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < RM; ++i)
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) acc[i][jj] = cmake((T)0, (T)0);
-    for (int64_t c = 0; c < nch; ++c) {
-        __syncthreads();   // the previous chunk's arithmetic is done with As / Bs
-#pragma unroll
-        for (int r = 0; r < RA; ++r) {
-            const int i = tid + r * kThreads;
-            As[i / TM][i % TM] = cscale(ra[r], sA);
+        for (int jj = 0; jj < RN; ++jj) acc[i][jj] = cmake((T)0, (T)0);
+    int slot = 1;   // of chunk c + 1
+#pragma unroll 1
+    for (int32_t c = 0; c < nch; ++c) {
+        const int ahead = slot == 2 ? 0 : slot + 1;
+        if (c + 2 < nch) koffs(c + 2, ahead);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();   // chunk c is there, and chunk c - 1's stage is free
+        if (c + 1 < nch) gather((c + 1) & 1, slot);
+        slot = ahead;
+        C *cur = As + (c & 1) * stage;
+        if (!late) {
+            const T sA = pow2<T>(-eA), sB = pow2<T>(-eB);
+#pragma unroll 1
+            for (int i = tid; i < stage; i += kThreads) cur[i] = cscale(cur[i], i < KC * PA ? sA : sB);
+            __syncthreads();
         }
+        const C *Ak = cur + ks * TK * PA + ty, *Bk = cur + KC * PA + ks * TK * PB + tx;
 #pragma unroll
-        for (int r = 0; r < RB; ++r) {
-            const int i = tid + r * kThreads;
-            Bs[i / TN][i % TN] = cscale(rb[r], sB);
+        for (int kk = 0; kk < TK; ++kk) {
+            C a[RM], b[RN];
+#pragma unroll
+            for (int i = 0; i < RM; ++i) a[i] = Ak[kk * PA + TY * i];
+#pragma unroll
+            for (int jj = 0; jj < RN; ++jj) b[jj] = Bk[kk * PB + TX * jj];
+#pragma unroll
+            for (int i = 0; i < RM; ++i)
+#pragma unroll
+                for (int jj = 0; jj < RN; ++jj) cfma(acc[i][jj], a[i], b[jj]);
         }
-        if (c + 1 < nch) koffs(c + 1);
-        __syncthreads();
-        if (c + 1 < nch) gather(c + 1);
+    }
+    if (late) {
+        const T s = pow2<T>(-eA - eB);
 #pragma unroll
-        for (int kk = 0; kk < kTileK; ++kk) {
-            C a[4], b[4];
+        for (int i = 0; i < RM; ++i)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + TY * i];
+            for (int jj = 0; jj < RN; ++jj) acc[i][jj] = cscale(acc[i][jj], s);
+    }
+    if constexpr (KS > 1) {   // upper half of the groups into the lower one, halving
+        C *P = reinterpret_cast<C *>(smem);
 #pragma unroll
-            for (int jj = 0; jj < 4; ++jj) b[jj] = Bs[kk][tx + TX * jj];
+        for (int h = KS / 2; h > 0; h /= 2) {
+            __syncthreads();
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < RM; ++i)
 #pragma unroll
-                for (int jj = 0; jj < 4; ++jj) cfma(acc[i][jj], a[i], b[jj]);
+                for (int jj = 0; jj < RN; ++jj)
+                    if (ks >= h && ks < 2 * h) P[(((ks - h) * RM + i) * RN + jj) * (TX * TY) + tid % (TX * TY)] = acc[i][jj];
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < RM; ++i)
+#pragma unroll
+                for (int jj = 0; jj < RN; ++jj)
+                    if (ks < h) {
+                        const C v = P[((ks * RM + i) * RN + jj) * (TX * TY) + tid % (TX * TY)];
+                        acc[i][jj].x += v.x;
+                        acc[i][jj].y += v.y;
+                    }
         }
     }
     float mx = 0.f;
+    if (ks == 0) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int64_t m = m0 + ty + TY * i;
-        if (m >= M) continue;
+        for (int i = 0; i < RM; ++i) {
+            const int64_t m = m0 + ty + TY * i;
+            if (m >= M) continue;
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-            int64_t n = n0 + tx + TX * jj;
-            if (n < N) {
-                Cp[m * N + n] = acc[i][jj];
-                mx = fmaxf(mx, absmax2(acc[i][jj]));
+            for (int jj = 0; jj < RN; ++jj) {
+                const int64_t n = n0 + tx + TX * jj;
+                if (n < N) {
+                    Cp[m * N + n] = acc[i][jj];
+                    mx = fmaxf(mx, absmax2(acc[i][jj]));
+                }
             }
         }
     }
@@ -1071,12 +1135,12 @@ __device__ __forceinline__ void run_tile(const StepDesc &d, int64_t tile, const 
         case STEP_ROWS: tile_rows_dispatch<T>(d, tile, j, smem, red, dyn); break;
         case STEP_TILE:
             if constexpr (sizeof(T) == 4) {
-                if (d.tile_rows == kTileNarrow) {
-                    tile_gemm<T, 2 * kTileM, kTileN / 2>(d, tile, j, smem, red);
-                    break;
-                }
+                if (d.tile_rows == TILE_NARROW) tile_gemm<T, 128, 32, 4, 4, 8, 1>(d, tile, j, smem, red);
+                else if (d.tile_rows == TILE_LONG_K) tile_gemm<T, 16, 16, 2, 2, 8, 4>(d, tile, j, smem, red);
+                else tile_gemm<T, 64, 64, 4, 4, 8, 1>(d, tile, j, smem, red);
+            } else {
+                tile_gemm<T, 32, 32, 2, 2, 8, 1>(d, tile, j, smem, red);
             }
-            tile_gemm<T, kTileM, kTileN>(d, tile, j, smem, red);
             break;
         case STEP_DOTP: tile_dotp<T>(d, tile, j, smem, dyn); break;
         case STEP_DOTF: tile_dotf<T>(d, j, smem); break;

@@ -463,3 +463,30 @@ def test_staged_step_shapes(tnsa, shape, tail, magnitude):
     # one rounding per leaf and stored step, two per term of a sum of K (or N, 2) complex products, 16 in the dot
     eps = (2 * (K + 2 + (N if tail else 0)) + 24) * 2.0 ** -24
     assert abs(out[0] - value(*tensors)) <= eps * value(*(np.abs(t) for t in tensors))
+
+
+# register-tiled steps: sizes around the tiles (64 x 64, 128 x 32, 16 x 16 with the shared index split, 32 x 32 in
+# complex128), both contiguities of each operand, entries so large or small that the scales move to the operands
+@pytest.mark.parametrize("shape", [(64, 64, 65), (65, 63, 129), (200, 70, 300), (129, 33, 70), (300, 31, 100), (8, 8, 512),
+                                   (17, 5, 300), (64, 16, 256), (15, 16, 1000), (2048, 33, 3), (1024, 4, 65)])
+@pytest.mark.parametrize("transposed", [(0, 0), (1, 0), (0, 1)])
+@pytest.mark.parametrize("precision,magnitude", [("c64", 1.0), ("c64", 2.0 ** 60), ("c64", 2.0 ** -60), ("c128", 1.0)])
+def test_register_tiled_step_shapes(tnsa, shape, transposed, precision, magnitude):
+    M, N, K = shape
+    rng = np.random.default_rng(M + N + K)
+
+    def normal(*s):
+        return (rng.standard_normal(s) + 1j * rng.standard_normal(s)) / math.sqrt(2)
+    a, b, c = normal(M, K) * magnitude, normal(K, N), normal(N, M)
+    ta, tb = transposed
+    edges = [(0, 0 if ta else 1, 1, 1 if tb else 0), (1, 0 if tb else 1, 2, 0), (2, 1, 0, 1 if ta else 0)]
+    net = tni.Network([a.T.copy() if ta else a, b.T.copy() if tb else b, c], np.array(edges, np.int32),
+                      np.zeros(3, np.int32), ["t"] * 3)
+    h = tnsa.tn_build(net)
+    ctx = tnsa.tn_ctx_create(0)
+    tnsa.tn_ctx_set_config(ctx, local_budget=0)
+    m, e, _ = tnsa.tn_contract(ctx, h, tnsa.tn_plan_import(h, [(0, 1), (3, 2)]), precision)
+    ref = np.einsum("ij,ji->", a @ b, c)
+    scale = np.einsum("ij,ji->", np.abs(a) @ np.abs(b), np.abs(c))
+    # two roundings per term of the complex sum over K, the leaves, the stored step and 16 in the closing dot
+    assert abs(m * 2.0 ** e - ref) <= (2 * K + 24) * (2.0 ** -24 if precision == "c64" else 2.0 ** -53 * 4) * scale
