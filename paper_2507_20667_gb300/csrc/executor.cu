@@ -124,6 +124,7 @@ struct tn_batch {
     // (gev, the last replay's); the ring then holds only a start and an end event per run
     cudaGraphExec_t pgexec = nullptr;
     std::vector<cudaEvent_t> gev;
+    std::vector<int32_t> gev_of;      // per slot boundary its event in gev: empty slots record none
     bool replay = false;
     int64_t runs = 0;
     // pending tensor updates (tn_batch_set_tensors): headers {dst element offset, count, src
@@ -1281,19 +1282,32 @@ cudaError_t enqueue_persistent(tn_batch *b, cudaStream_t st, std::vector<cudaEve
     e = ensure_events(ev, 3 + 3 * b->phases.size());
     if (e != cudaSuccess) return e;
     size_t k = 0;
-    e = cudaEventRecordWithFlags(ev[k++], st, rec_flags);
+    if (capturing) b->gev_of.clear();
+    // every boundary of a direct run; in a recorded one a node costs about 2 us per replay, and the
+    // boundary after an empty slot shares the event before it
+    auto record = [&](bool ran) {
+        if (capturing) {
+            if (!ran) {
+                b->gev_of.push_back(b->gev_of.back());
+                return cudaSuccess;
+            }
+            b->gev_of.push_back((int32_t)k);
+        }
+        return cudaEventRecordWithFlags(ev[k++], st, rec_flags);
+    };
+    e = record(true);
     if (e == cudaSuccess) {
         t_enqueue_stage = "warp programs";
         e = launch_local(b->c128, b->d_jobs, b->d_local, b->n_warp_items, 0, 0, b->dyn_smem, b->dyn_big,
                          b->d_prof, st);
     }
-    if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev[k++], st, rec_flags);
+    if (e == cudaSuccess) e = record(b->n_warp_items > 0);
     if (e == cudaSuccess) {
         t_enqueue_stage = "subtree programs";
         e = launch_local(b->c128, b->d_jobs, b->d_local + b->n_warp_items, 0, b->n_block_items, b->n_big_items,
                          b->dyn_smem, b->dyn_big, b->d_prof, st);
     }
-    if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev[k++], st, rec_flags);
+    if (e == cudaSuccess) e = record(b->n_block_items + b->n_big_items > 0);
     const bool tf32 = b->prec == TN_TF32_SPLIT;
     for (size_t p = 0; e == cudaSuccess && p < b->phases.size(); ++p) {
         const tn_batch::Phase &ph = b->phases[p];
@@ -1302,19 +1316,19 @@ cudaError_t enqueue_persistent(tn_batch *b, cudaStream_t st, std::vector<cudaEve
             t_enqueue_stage = "tensor-core operand packing";
             e = launch_tc_pack(tf32, b->d_jobs, b->d_pack + ph.pack0, ph.n_pack, st);
         }
-        if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev[k++], st, rec_flags);
+        if (e == cudaSuccess) e = record(ph.n_pack > 0);
         if (e == cudaSuccess && ph.n_gemm > 0) {
             t_enqueue_stage = "tensor-core GEMM";
             e = launch_tc_gemm(tf32, b->d_jobs, b->d_gemm + ph.gemm0, ph.n_gemm, reinterpret_cast<int32_t *>(cnt + 2),
                                b->wait_ns, st);
         }
-        if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev[k++], st, rec_flags);
+        if (e == cudaSuccess) e = record(ph.n_gemm > 0);
         if (e == cudaSuccess && ph.n_work > 0) {
             t_enqueue_stage = "dataflow kernel";
             e = launch_persistent(b->c128, b->d_jobs, b->d_work + ph.work0, ph.n_work, cnt, b->grid, b->wait_ns,
                                   b->d_prof, st);
         }
-        if (e == cudaSuccess) e = cudaEventRecordWithFlags(ev[k++], st, rec_flags);
+        if (e == cudaSuccess) e = record(ph.n_work > 0);
     }
     return e;
 }
@@ -2269,11 +2283,12 @@ tn_status tn_batch_kernel_times(const tn_batch *b, int32_t n_runs, double *mean_
     if (b->replay) n_runs = 1;   // the graph's events time its last replay
     for (int64_t r = b->runs - n_runs; r < b->runs; ++r) {
         const std::vector<cudaEvent_t> &ev = b->replay ? b->gev : b->kev[r % tn_batch::kRing];
-        if (ev.size() < n_ev) return fail(TN_EINVAL, "no timing of that run");
-        CK(cudaEventSynchronize(ev[n_ev - 1]));
+        if (ev.size() < n_ev || (b->replay && b->gev_of.size() != n_ev)) return fail(TN_EINVAL, "no timing of that run");
+        auto at = [&](size_t i) { return ev[b->replay ? (size_t)b->gev_of[i] : i]; };
+        CK(cudaEventSynchronize(at(n_ev - 1)));
         for (size_t i = 0; i + 1 < n_ev; ++i) {
             float ms = 0;
-            CK(cudaEventElapsedTime(&ms, ev[i], ev[i + 1]));
+            if (at(i) != at(i + 1)) CK(cudaEventElapsedTime(&ms, at(i), at(i + 1)));
             // slots: 0 warp programs, 1 block and large programs, then (pack, GEMM, dataflow) per phase
             const int cls = i < 2 ? (int)i : 2 + (int)((i - 2) % 3);
             acc[cls] += ms;

@@ -4,11 +4,13 @@
 namespace tn {
 
 cudaError_t launch_persistent_f32(const JobPtrs *jobs_dev, const WorkItem *work, int64_t n_work, uint32_t *counter,
-                                  int32_t grid, long long wait_ns, long long *prof, cudaStream_t stream) {
+                                  int32_t grid, int32_t first_wave, long long wait_ns, long long *prof,
+                                  cudaStream_t stream) {
     auto kern = prof ? k_persist<float, true> : k_persist<float, false>;
     const cudaError_t e = allow_dyn_smem(kern, kPersistDynSmem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)grid, kThreads, kPersistDynSmem, stream>>>(jobs_dev, work, n_work, counter, wait_ns, prof);
+    kern<<<(unsigned)grid, kThreads, kPersistDynSmem, stream>>>(jobs_dev, work, n_work, counter, first_wave, wait_ns,
+                                                                   prof);
     return cudaGetLastError();
 }
 

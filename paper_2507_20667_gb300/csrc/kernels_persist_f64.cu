@@ -21,13 +21,17 @@ cudaError_t launch_persistent(bool c128, const JobPtrs *jobs_dev, const WorkItem
                               uint32_t *counter, int32_t grid, long long wait_ns, long long *prof,
                               cudaStream_t stream) {
     if (n_work <= 0) return cudaSuccess;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
     if (grid > n_work) grid = (int32_t)n_work;
-    if (!c128) return launch_persistent_f32(jobs_dev, work, n_work, counter, grid, wait_ns, prof, stream);
+    if (!c128) return launch_persistent_f32(jobs_dev, work, n_work, counter, grid, sms, wait_ns, prof, stream);
     if (prof)
-        k_persist<double, true><<<(unsigned)grid, kThreads, 0, stream>>>(jobs_dev, work, n_work, counter, wait_ns,
+        k_persist<double, true><<<(unsigned)grid, kThreads, 0, stream>>>(jobs_dev, work, n_work, counter, sms, wait_ns,
                                                                         prof);
     else
-        k_persist<double, false><<<(unsigned)grid, kThreads, 0, stream>>>(jobs_dev, work, n_work, counter, wait_ns,
+        k_persist<double, false><<<(unsigned)grid, kThreads, 0, stream>>>(jobs_dev, work, n_work, counter, sms, wait_ns,
                                                                          nullptr);
     return cudaGetLastError();
 }

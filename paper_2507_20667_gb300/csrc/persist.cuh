@@ -20,7 +20,7 @@ namespace {
 template <typename T, bool PROF>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1)
     k_persist(const JobPtrs *__restrict__ jobs, const WorkItem *__restrict__ work, int64_t n_work,
-              uint32_t *counter, long long wait_ns, long long *prof) {
+              uint32_t *counter, int32_t first_wave, long long wait_ns, long long *prof) {
     int32_t *abort_flag = reinterpret_cast<int32_t *>(counter + 1);
     extern __shared__ __align__(16) char dyn[];
     __shared__ __align__(16) StepDesc d;
@@ -34,8 +34,14 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1)
     // trip is off the critical path.  A block claims items in increasing order and runs them in
     // that order; the earliest unfinished item is therefore always being run (never only held),
     // which keeps the list order deadlock-free.
+    // With fewer items than two per block, the blocks past the first one of each SM claim a moment
+    // later, so that the first items -- the heaviest paths -- do not share an SM while others idle
+    // (chains of 64 24-qubit amplitudes: 214 k cycles two to an SM, 150 k one to an SM).
     uint32_t nxt = 0;
-    if (threadIdx.x == 0) nxt = atomicAdd(counter, 1u);
+    if (threadIdx.x == 0) {
+        if ((int32_t)blockIdx.x >= first_wave && n_work < 2 * (int64_t)gridDim.x) __nanosleep(1000);
+        nxt = atomicAdd(counter, 1u);
+    }
     while (true) {
         if (threadIdx.x == 0) s_item = nxt;
         __syncthreads();
@@ -95,7 +101,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1)
 
 // complex64 instantiation (kernels_persist_f32.cu)
 cudaError_t launch_persistent_f32(const JobPtrs *jobs_dev, const WorkItem *work, int64_t n_work, uint32_t *counter,
-                                  int32_t grid, long long wait_ns, long long *prof, cudaStream_t stream);
+                                  int32_t grid, int32_t first_wave, long long wait_ns, long long *prof,
+                                  cudaStream_t stream);
 int32_t persistent_blocks_per_sm_f32();
 
 }  // namespace tn

@@ -252,3 +252,27 @@ def test_staged_updates_accumulate_and_alternate(tnsa):
             ref = psi[tuple(x)]
             if abs(ref) >= 1e-3 * 2.0 ** -6:
                 check(got[i], ref, TOL["c64"], f"round {rnd} job {i}")
+
+
+@pytest.mark.parametrize("sizes", [(65, 71), (64, 129), (1001, 2047), (4096, 4097)])
+def test_large_leaves_at_any_alignment(sizes):
+    """Dense leaves of odd and even sizes, several jobs (whose leaves then start at odd offsets): every
+    job's closing dots equal numpy's."""
+    from paper_2507_20667_gb300 import tnsa
+    rng = np.random.default_rng(sum(sizes))
+    nets, refs, scales = [], [], []
+    for _ in range(3):
+        t = [rng.standard_normal(n) + 1j * rng.standard_normal(n) for n in sizes for _ in range(2)]
+        nets.append(tni.Network(t, np.array([(0, 0, 1, 0), (2, 0, 3, 0)], np.int32), np.zeros(4, np.int32), ["t"] * 4))
+        refs.append((t[0] * t[1]).sum() * (t[2] * t[3]).sum())
+        scales.append(np.abs(t[0] * t[1]).sum() * np.abs(t[2] * t[3]).sum())
+    hs = [tnsa.tn_build(n) for n in nets]
+    plan = tnsa.tn_plan_import(hs[0], [(0, 1), (2, 3), (4, 5)])
+    ctx = tnsa.tn_ctx_create(0)
+    tnsa.tn_ctx_set_config(ctx, local_budget=0)
+    b = tnsa.tn_batch_create(ctx, hs, [plan] * 3, "c64")
+    tnsa.tn_batch_run(b)
+    m, e, st = tnsa.tn_batch_results(b)
+    assert (st == 0).all()
+    # leaves, products, bursts of 16 products and the stored dots are rounded to 24 bits
+    assert (np.abs(m * np.exp2(e) - refs) <= 2 * 24 * 2.0 ** -24 * np.array(scales)).all()
