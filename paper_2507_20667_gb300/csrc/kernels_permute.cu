@@ -4,7 +4,6 @@
 // the buffers are aligned for it.  One kernel then moves tiles: see TilePerm.
 #include <algorithm>
 #include <cstdint>
-#include <vector>
 
 #include "kernels.cuh"
 
@@ -194,24 +193,30 @@ __global__ void __launch_bounds__(256) k_perm_tile(const E *__restrict__ in, E *
 // Builds the tiles of plan p: runs of about `edge` elements on both sides, at most `area` elements.
 // false if the tensor has too many of them.
 bool tile_perm(const PermPlan &p, int32_t edge, int32_t area, TilePerm &g) {
-    std::vector<char> used(p.rank, 0);
-    std::vector<int32_t> by_in(p.rank);  // axes by increasing input stride
+    // fixed arrays: a small permutation costs little more than its launch
+    char used[kMaxRank] = {};
+    int32_t by_in[kMaxRank];  // axes by increasing input stride
     for (int32_t t = 0; t < p.rank; ++t) by_in[t] = t;
-    std::sort(by_in.begin(), by_in.end(), [&](int32_t x, int32_t y) { return p.istride[x] < p.istride[y]; });
+    std::sort(by_in, by_in + p.rank, [&](int32_t x, int32_t y) { return p.istride[x] < p.istride[y]; });
     struct Axis { int64_t dim, in, out; };
-    std::vector<Axis> A, B, C, R;
+    struct Axes {
+        Axis a[kMaxRank + 4];
+        int32_t n = 0;
+        void push_back(const Axis &x) { a[n++] = x; }
+        Axis &back() { return a[n - 1]; }
+    } A, B, C, R;
     // an edge of at most t splits n indices into chunks of equal length
     auto chunk = [](int64_t n, int64_t t) {
         const int64_t c = (n + t - 1) / t;
         return (n + c - 1) / c;
     };
-    auto prod = [](const std::vector<Axis> &v) {
+    auto prod = [](const Axes &v) {
         int64_t x = 1;
-        for (const Axis &a : v) x *= a.dim;
+        for (int32_t i = 0; i < v.n; ++i) x *= v.a[i].dim;
         return x;
     };
     int32_t ia = p.rank - 1, ib = 0;
-    auto take = [&](std::vector<Axis> &v, int32_t t) {
+    auto take = [&](Axes &v, int32_t t) {
         v.push_back({p.odim[t], p.istride[t], p.ostride[t]});
         used[t] = 1;
     };
@@ -232,15 +237,15 @@ bool tile_perm(const PermPlan &p, int32_t edge, int32_t area, TilePerm &g) {
         g.before[q] = 1;
     }
     // cuts the last axis of a group so that its extent is at most lim
-    auto cut = [&](std::vector<Axis> &v, int64_t lim, int q) {
-        if (v.empty()) return;
+    auto cut = [&](Axes &v, int64_t lim, int q) {
+        if (v.n == 0) return;
         Axis &last = v.back();
         const int64_t before = prod(v) / last.dim, len = chunk(last.dim, std::max<int64_t>(1, lim / before));
         if (len < last.dim) {
             R.push_back({(last.dim + len - 1) / len, last.in * len, last.out * len});
             g.cutdim[q] = last.dim;
             g.cutlen[q] = (int32_t)len;
-            g.cut[q] = (int32_t)R.size() - 1;   // index into R, renumbered below
+            g.cut[q] = R.n - 1;   // index into R, renumbered below
             g.before[q] = (int32_t)before;
             last.dim = len;
         }
@@ -286,24 +291,28 @@ bool tile_perm(const PermPlan &p, int32_t edge, int32_t area, TilePerm &g) {
     g.mi = magic(ti);
     g.ma = magic(ta);
     g.mb = magic(tb);
-    g.na = (int32_t)A.size();
-    g.nb = (int32_t)B.size();
-    g.nc = (int32_t)C.size();
-    for (int32_t i = 0; i < g.na; ++i) { g.adim[i] = (int32_t)A[i].dim; g.ain[i] = A[i].in; }
-    for (int32_t i = 0; i < g.nb; ++i) { g.bdim[i] = (int32_t)B[i].dim; g.bout[i] = B[i].out; }
-    for (int32_t i = 0; i < g.nc; ++i) { g.cdim[i] = (int32_t)C[i].dim; g.cin[i] = C[i].in; g.cout[i] = C[i].out; }
+    g.na = A.n;
+    g.nb = B.n;
+    g.nc = C.n;
+    for (int32_t i = 0; i < g.na; ++i) { g.adim[i] = (int32_t)A.a[i].dim; g.ain[i] = A.a[i].in; }
+    for (int32_t i = 0; i < g.nb; ++i) { g.bdim[i] = (int32_t)B.a[i].dim; g.bout[i] = B.a[i].out; }
+    for (int32_t i = 0; i < g.nc; ++i) {
+        g.cdim[i] = (int32_t)C.a[i].dim;
+        g.cin[i] = C.a[i].in;
+        g.cout[i] = C.a[i].out;
+    }
     // the tile index: chunk numbers and the other axes, innermost in the output first, so that
     // consecutive tiles write neighbouring runs
     for (int32_t t = 0; t < p.rank; ++t)
         if (!used[t]) R.push_back({p.odim[t], p.istride[t], p.ostride[t]});
-    std::vector<int32_t> ord(R.size());
-    for (size_t i = 0; i < ord.size(); ++i) ord[i] = (int32_t)i;
-    std::sort(ord.begin(), ord.end(), [&](int32_t x, int32_t y) { return R[x].out < R[y].out; });
-    g.nr = (int32_t)R.size();
+    int32_t ord[kMaxRank + 4];
+    for (int32_t i = 0; i < R.n; ++i) ord[i] = i;
+    std::sort(ord, ord + R.n, [&](int32_t x, int32_t y) { return R.a[x].out < R.a[y].out; });
+    g.nr = R.n;
     int64_t tiles = 1;
     int32_t cuts[4] = {-1, -1, -1, -1};
     for (int32_t i = 0; i < g.nr; ++i) {
-        const Axis &x = R[ord[i]];
+        const Axis &x = R.a[ord[i]];
         g.rbelow[i] = (uint32_t)tiles;
         if (x.dim > 0x7fffffffLL || tiles > 0x7fffffffLL / x.dim) return false;
         tiles *= x.dim;
@@ -338,46 +347,48 @@ cudaError_t perm_launch(const void *src, void *dst, const PermPlan &p, cudaStrea
     E *out = static_cast<E *>(dst);
     constexpr int AREA = sizeof(E) <= 8 ? 2048 : 1024;
     TilePerm g;
-    if (p.total <= 0x7fffffffLL) {
+    auto ragged = [&]() {
+        bool r = false;
+        for (int q = 0; q < 4; ++q) r = r || (g.cut[q] >= 0 && g.cutdim[q] % g.cutlen[q] != 0);
+        return r;
+    };
+    const bool wide = p.total > 0x7fffffffLL;
+    if (!wide && p.total > 152 * 6 * 1024) {   // enough tiles to choose their size
         if (!tile_perm(p, kTileEdge, AREA, g)) return cudaErrorInvalidValue;
-        bool ragged = false;
-        for (int q = 0; q < 4; ++q) ragged = ragged || (g.cut[q] >= 0 && g.cutdim[q] % g.cutlen[q] != 0);
-        if (!ragged) return launch_tiles<E, AREA / 256, false, int32_t>(in, out, g, st);
+        if (!ragged()) return launch_tiles<E, AREA / 256, false, int32_t>(in, out, g, st);
     }
     if (!tile_perm(p, kTileEdge, 1024, g)) return cudaErrorInvalidValue;
-    if (p.total <= 0x7fffffffLL) return launch_tiles<E, 4, true, int32_t>(in, out, g, st);
-    return launch_tiles<E, 4, true, int64_t>(in, out, g, st);
+    if (wide) return launch_tiles<E, 4, true, int64_t>(in, out, g, st);
+    return ragged() ? launch_tiles<E, 4, true, int32_t>(in, out, g, st)
+                    : launch_tiles<E, 4, false, int32_t>(in, out, g, st);
 }
 
 // The fused plan of a permutation; false if it has too many axes.
 bool perm_plan(int32_t rank, const int64_t *dims, const int32_t *perm, PermPlan &p) {
-    // input strides
-    std::vector<int64_t> istr(rank);
+    // input strides (rank <= kMaxRank)
+    if (rank > kMaxRank) return false;
+    int64_t istr[kMaxRank];
     int64_t acc = 1;
     for (int32_t t = rank - 1; t >= 0; --t) { istr[t] = acc; acc *= dims[t]; }
     p = PermPlan{};
     p.total = acc;
     p.inner = 1;
     // output axes (dims of 1 dropped), fused when adjacent in the input in the same order
-    std::vector<int64_t> od, is;
+    int64_t od[kMaxRank], is[kMaxRank];
+    int32_t n = 0;
     for (int32_t t = 0; t < rank; ++t) {
-        int64_t d = dims[perm[t]], s = istr[perm[t]];
+        const int64_t d = dims[perm[t]], s = istr[perm[t]];
         if (d == 1) continue;
-        if (!od.empty() && is.back() == d * s) {
-            od.back() *= d;
-            is.back() = s;
+        if (n && is[n - 1] == d * s) {
+            od[n - 1] *= d;
+            is[n - 1] = s;
         } else {
-            od.push_back(d);
-            is.push_back(s);
+            od[n] = d;
+            is[n++] = s;
         }
     }
-    if (!od.empty() && is.back() == 1) {
-        p.inner = od.back();
-        od.pop_back();
-        is.pop_back();
-    }
-    p.rank = (int32_t)od.size();
-    if (p.rank > kMaxRank) return false;
+    if (n && is[n - 1] == 1) p.inner = od[--n];
+    p.rank = n;
     acc = p.inner;
     for (int32_t t = p.rank - 1; t >= 0; --t) {
         p.odim[t] = od[t];
