@@ -2203,11 +2203,18 @@ tn_status tn_batch_set_tensors(tn_batch *b, int32_t count, const int32_t *job, c
     if (count < 0) return fail(TN_EINVAL, "count must be >= 0");
     // validate everything first: a rejected call stages nothing
     size_t n_val = 0;
+    int32_t last = -1, n_leaves = 0;   // the job of the previous update, its structure's leaves
+    const int64_t *leaf_off = nullptr;
     for (int32_t i = 0; i < count; ++i) {
-        if (job[i] < 0 || job[i] >= b->n_jobs) return fail(TN_EINVAL, "job index out of range");
-        const Compiled &c = b->comp[b->job_comp[job[i]]];
-        if (tensor[i] < 0 || tensor[i] >= c.n) return fail(TN_EINVAL, "tensor index out of range");
-        n_val += 2 * (size_t)(c.leaf_off[tensor[i] + 1] - c.leaf_off[tensor[i]]);
+        if (job[i] != last) {
+            if (job[i] < 0 || job[i] >= b->n_jobs) return fail(TN_EINVAL, "job index out of range");
+            last = job[i];
+            const Compiled &c = b->comp[b->job_comp[last]];
+            n_leaves = c.n;
+            leaf_off = c.leaf_off.data();
+        }
+        if (tensor[i] < 0 || tensor[i] >= n_leaves) return fail(TN_EINVAL, "tensor index out of range");
+        n_val += 2 * (size_t)(leaf_off[tensor[i] + 1] - leaf_off[tensor[i]]);
     }
     if (count == 0) return TN_OK;
     if (!entries_in_range(data, n_val))
@@ -2222,18 +2229,20 @@ tn_status tn_batch_set_tensors(tn_batch *b, int32_t count, const int32_t *job, c
     if (s == TN_OK) s = pinned_reserve(sg.val, sg.val.size + sizeof(double) * n_val);
     if (s != TN_OK) return s;
     int64_t *hdr = reinterpret_cast<int64_t *>(sg.hdr.p + sg.hdr.size);
-    double *val = reinterpret_cast<double *>(sg.val.p + sg.val.size);
     int64_t vpos = (int64_t)(sg.val.size / (2 * sizeof(double)));   // complex entries staged so far
-    size_t src = 0;
+    std::memcpy(sg.val.p + sg.val.size, data, sizeof(double) * n_val);   // back to back in the updates' order
+    last = -1;
+    int64_t base = 0;
     for (int32_t i = 0; i < count; ++i) {
-        const Compiled &c = b->comp[b->job_comp[job[i]]];
-        const int64_t off = c.leaf_off[tensor[i]], cnt = c.leaf_off[tensor[i] + 1] - off;
-        hdr[3 * i] = b->leaf64_off[job[i]] + off;
+        if (job[i] != last) {
+            last = job[i];
+            leaf_off = b->comp[b->job_comp[last]].leaf_off.data();
+            base = b->leaf64_off[last];
+        }
+        const int64_t off = leaf_off[tensor[i]], cnt = leaf_off[tensor[i] + 1] - off;
+        hdr[3 * i] = base + off;
         hdr[3 * i + 1] = cnt;
         hdr[3 * i + 2] = vpos;
-        std::memcpy(val, data + src, sizeof(double) * 2 * (size_t)cnt);
-        val += 2 * cnt;
-        src += 2 * (size_t)cnt;
         vpos += cnt;
     }
     sg.hdr.size += 3 * sizeof(int64_t) * (size_t)count;

@@ -1,7 +1,9 @@
 // Tile-level device functions of the contraction kernels.  One call computes one work tile of
 // one step; the per-step kernels map blocks to tiles, the persistent kernel claims tiles from a
-// global work list.  All operand loads bypass L1 (ld.global.cg): inside one persistent launch an
-// arena address is rewritten by later steps, so an SM must never see a stale L1 line.
+// global work list.  Inside one persistent launch an arena address is rewritten by later steps, so an SM
+// must never see a stale L1 line: operand loads bypass L1 (ld.global.cg), or, where only 8-byte
+// asynchronous copies fit (which pass through L1), come after the block's wait for the operand's producer,
+// an acquire at GPU scope, or read leaves and program results, complete before the launch.
 #pragma once
 
 #include <cstdint>

@@ -3,6 +3,7 @@
 
 #include <array>
 #include <cstdint>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -24,9 +25,22 @@ inline tn_u128 to_abi(u128 x) { return tn_u128{(uint64_t)x, (uint64_t)(x >> 64)}
 // tracks each tensor's max-abs in FP32, so larger leaf entries (possible only in complex128) would
 // saturate it; intermediates of any size are fine (every step rescales its operands).
 constexpr double kMaxEntry = 170141183460469231731687303715884105728.0;   // 2^127
+// (by their bits: the magnitudes of finite doubles order like their bit patterns, infinities and NaN
+// lie above; whole blocks are tested without a branch per entry)
 inline bool entries_in_range(const double *p, size_t n) {
-    for (size_t i = 0; i < n; ++i)
-        if (!(p[i] < kMaxEntry && p[i] > -kMaxEntry)) return false;   // NaN fails both
+    uint64_t limit;
+    const double top = kMaxEntry;
+    std::memcpy(&limit, &top, sizeof(limit));
+    for (size_t i = 0; i < n;) {
+        const size_t e = i + 512 < n ? i + 512 : n;
+        uint64_t bad = 0;
+        for (; i < e; ++i) {
+            uint64_t b;
+            std::memcpy(&b, p + i, sizeof(b));
+            bad |= (uint64_t)((b & 0x7fffffffffffffffull) >= limit);
+        }
+        if (bad) return false;
+    }
     return true;
 }
 
