@@ -270,7 +270,7 @@ tn_status tn_ctx_set_local_budget(tn_ctx *ctx, int32_t bytes);
  *   warp_programs    1: warp programs -- subtrees of small steps run by one warp each; 0: none
  *   tc_min_m/n/k     in the split precisions, a dense step runs on the tensor cores when
  *                    M >= tc_min_m, N >= tc_min_n and K >= tc_min_k
- *   rows_chains      1: a chain of narrow dataflow steps, each consuming the previous one's output
+ *   rows_chains      1: a chain of dataflow steps that fit shared memory, each consuming the previous one's output
  *                    as its large operand, runs in one block of the persistent kernel with the
  *                    tensor kept in shared memory between the steps (complex64 storage); 0: every
  *                    step writes its output to the arena.  Results are bit-identical either way.
