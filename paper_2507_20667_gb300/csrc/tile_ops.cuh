@@ -692,7 +692,10 @@ __device__ __forceinline__ int32_t rows_chain(const StepDesc &d, const JobPtrs &
     while (true) {
         const StepHead &cur = ring[at];
         const int32_t after = at == 2 ? 0 : at + 1;
-        const StepHead *next = cur.chain_next >= 0 ? ring + after : nullptr;
+        // read here: past the step's last barrier the head's place belongs to the copy of the step after
+        // the next one, which other lanes may have started
+        const int32_t cont = cur.chain_next;
+        const StepHead *next = cont >= 0 ? ring + after : nullptr;
         uint32_t next_max = 0;
         int32_t next_exp = 0;
         if (next) {
@@ -707,7 +710,7 @@ __device__ __forceinline__ int32_t rows_chain(const StepDesc &d, const JobPtrs &
             if (threadIdx.x == 0) j.exp2[cur.node_c] = xc;
             return n;
         }
-        if (threadIdx.x == 0) chain[n] = cur.chain_next;
+        if (threadIdx.x == 0) chain[n] = cont;
         ++n;
         at = after;
         xa = xc;

@@ -490,3 +490,42 @@ def test_register_tiled_step_shapes(tnsa, shape, transposed, precision, magnitud
     scale = np.einsum("ij,ji->", np.abs(a) @ np.abs(b), np.abs(c))
     # two roundings per term of the complex sum over K, the leaves, the stored step and 16 in the closing dot
     assert abs(m * 2.0 ** e - ref) <= (2 * K + 24) * (2.0 ** -24 if precision == "c64" else 2.0 ** -53 * 4) * scale
+
+
+# chains of `length` staged steps: from four on the ring of three step heads wraps around, past 32 the chain is cut
+@pytest.mark.parametrize("length", [3, 4, 5, 9, 40])
+@pytest.mark.parametrize("shape", [(512, 4), (512, 16), (256, 32)])
+def test_long_chains_of_staged_steps(tnsa, length, shape):
+    """Every step of a chain completes its own counter (a wrong one would leave a consumer waiting or let it
+    start early): many jobs, statuses, and the bits of the same steps run one by one."""
+    M, K = shape
+    rng = np.random.default_rng(length * 100 + K)
+
+    def normal(*s):
+        return rng.standard_normal(s) + 1j * rng.standard_normal(s)
+    nets = []
+    for _ in range(4):
+        mats = [np.linalg.qr(normal(K, K))[0] for _ in range(length)]
+        edges = [(0, 1, 1, 0)] + [(i, 1, i + 1, 0) for i in range(1, length + 2)] + [(length + 2, 1, 0, 0)]
+        nets.append(tni.Network([normal(M, 2), normal(2, K)] + mats + [normal(K, M)], np.array(edges, np.int32),
+                                np.zeros(length + 3, np.int32), ["t"] * (length + 3)))
+    hs = [tnsa.tn_build(n) for n in nets]
+    plan = tnsa.tn_plan_import(hs[0], [(0, 1)] + [(length + 3 + i, 2 + i) for i in range(length + 1)])
+    assert tnsa.tn_plan_compile_stats(hs[0], plan, "c64", 0)["n_chained"] == length - (length + 31) // 32
+    out = []
+    for chains in (1, 0):
+        c = tnsa.tn_ctx_create(0)
+        tnsa.tn_ctx_set_config(c, local_budget=0, rows_chains=chains)
+        b = tnsa.tn_batch_create(c, hs * 100, [plan] * 400, "c64")
+        tnsa.tn_batch_run(b)
+        m, e, st = tnsa.tn_batch_results(b)
+        assert (st == 0).all()
+        out.append((m, e))
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+    for i, n in enumerate(nets):
+        # a step rounds its B and its output once and sums K complex products: its error is at most 2 (K + 2) 2^-24
+        # of |A| |B|, whose norm is at most sqrt(K) times that of A (B is unitary); the dot adds 16 roundings
+        t = n.tensors
+        bound = (length * 2 * (K + 2) * math.sqrt(K) + 32) * 2.0 ** -24 * math.prod(map(np.linalg.norm, (t[0], t[1], t[-1])))
+        got = out[0][0][i::4] * np.exp2(out[0][1][i::4].astype(float))
+        assert (np.abs(got - np.trace(np.linalg.multi_dot(t))) <= bound).all()
