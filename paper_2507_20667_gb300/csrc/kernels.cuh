@@ -51,8 +51,9 @@ enum StepFlags : int32_t {
     FLAG_A_POW2 = 4096      // FLAG_A_SMEM: A's dims are powers of two (swizzled layout)
 };
 
-// The part of a step descriptor that staged steps need: their index maps are tabulated.
-struct StepHead {
+// The part of a step descriptor that staged steps need: their index maps are tabulated.  Descriptors and heads
+// are copied in 16-byte pieces, so every one of them, in shared memory too, is aligned for that.
+struct alignas(16) StepHead {
     int64_t M, N, K;
     int64_t a_off, b_off, c_off;   // element offsets into the leaf buffer or the arena
     int64_t img_a, img_b;          // TC: byte offsets in the arena of the packed operand images

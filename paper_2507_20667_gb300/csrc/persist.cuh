@@ -23,12 +23,12 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1)
               uint32_t *counter, int32_t first_wave, long long wait_ns, long long *prof) {
     int32_t *abort_flag = reinterpret_cast<int32_t *>(counter + 1);
     extern __shared__ __align__(16) char dyn[];
-    __shared__ __align__(16) StepDesc d;
+    __shared__ StepDesc d;
     __shared__ __align__(16) char smem[Scratch<T>::bytes];
     __shared__ float red[32];
     __shared__ uint32_t s_item;
     __shared__ int32_t s_ok;
-    __shared__ __align__(16) StepHead s_ring[3];   // heads of the current ROWS chain's steps
+    __shared__ StepHead s_ring[3];           // heads of the current ROWS chain's steps
     __shared__ int32_t s_chain[kMaxChain];   // continuation steps of the current ROWS chain
     // Claim-ahead: thread 0 claims the next item while the current one runs, so the claim's round
     // trip is off the critical path.  A block claims items in increasing order and runs them in

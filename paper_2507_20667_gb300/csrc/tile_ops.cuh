@@ -180,7 +180,9 @@ __device__ __forceinline__ void load_desc(StepDesc &dst, const StepDesc *src) {
         d[i] = __ldcg(s + i);
     __syncthreads();
 }
-static_assert(sizeof(StepDesc) % sizeof(int4) == 0, "descriptor must be a multiple of 16 bytes");
+static_assert(sizeof(StepDesc) % sizeof(int4) == 0 && alignof(StepDesc) % sizeof(int4) == 0 &&
+                  alignof(StepHead) % sizeof(int4) == 0,
+              "descriptors are copied in 16-byte pieces");
 
 // The same copy in two halves, so that the loads can be in flight while thread 0 waits on the
 // step's dependencies: desc_fetch issues them (one 16-byte piece per thread and round), desc_store
