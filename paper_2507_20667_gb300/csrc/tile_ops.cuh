@@ -508,7 +508,7 @@ __device__ float rows_smem_core(const StepHead &d, const JobPtrs &j, char *smem,
     if (!fold) {
         const float sA = pow2<float>(-eA);
 #pragma unroll 1
-        for (int32_t i = tid; i < (MK + 15) / 16 * 16; i += kThreads) As[i] = cscale(As[i], sA);
+        for (int32_t i = tid; i < MK; i += kThreads) As[i] = cscale(As[i], sA);   // swizzled or not: B may follow
         __syncthreads();
     }
     prof_phase<PROF>(prof, 7, tp);

@@ -529,3 +529,29 @@ def test_long_chains_of_staged_steps(tnsa, length, shape):
         bound = (length * 2 * (K + 2) * math.sqrt(K) + 32) * 2.0 ** -24 * math.prod(map(np.linalg.norm, (t[0], t[1], t[-1])))
         got = out[0][0][i::4] * np.exp2(out[0][1][i::4].astype(float))
         assert (np.abs(got - np.trace(np.linalg.multi_dot(t))) <= bound).all()
+
+
+# staged steps whose B lies behind A in shared memory (it does not fit the scratch area), M K no multiple of 16, an A
+# whose exponent is not 0, and a B near the ends of the FP32 range: A is then scaled where it lies
+@pytest.mark.parametrize("shape", [(101, 50, 45), (77, 33, 44), (126, 64, 45)])
+@pytest.mark.parametrize("magnitude", [1.0, 2.0 ** 100, 2.0 ** -100])
+def test_staged_step_scales_only_its_own_operand(tnsa, shape, magnitude):
+    M, N, K = shape
+    rng = np.random.default_rng(M + N + K)
+
+    def normal(*s):
+        return rng.standard_normal(s) + 1j * rng.standard_normal(s)
+
+    def exponent(t):
+        return int(np.frexp(max(np.abs(t.real).max(), np.abs(t.imag).max()))[1])
+    x, y, b, d = normal(M, 16), normal(16, K), normal(K, N) * magnitude, normal(M, N)
+    assert exponent((x * 2.0 ** -exponent(x)) @ (y * 2.0 ** -exponent(y))) != 0
+    net = tni.Network([x, y, b, d], np.array([(0, 1, 1, 0), (1, 1, 2, 0), (0, 0, 3, 0), (2, 1, 3, 1)], np.int32),
+                      np.zeros(4, np.int32), ["t"] * 4)
+    h = tnsa.tn_build(net)
+    c = tnsa.tn_ctx_create(0)
+    tnsa.tn_ctx_set_config(c, local_budget=0)
+    m, e, _ = tnsa.tn_contract(c, h, tnsa.tn_plan_import(h, [(0, 1), (4, 2), (5, 3)]), "c64")
+    ref, scale = ((x @ y @ b) * d).sum(), ((np.abs(x) @ np.abs(y) @ np.abs(b)) * np.abs(d)).sum()
+    # one rounding per leaf and stored step, two per term of the sums over 16 and K, 16 in the dot
+    assert abs(m * 2.0 ** e - ref) <= (2 * (K + 16) + 24) * 2.0 ** -24 * scale
