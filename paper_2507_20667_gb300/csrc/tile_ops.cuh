@@ -747,9 +747,11 @@ __device__ __forceinline__ void tile_rows_dispatch(const StepDesc &d, int64_t ti
 // in chunks of KS TK: the block's KS thread groups take TK shared indices of a chunk each (their sums are
 // added in a fixed order at the end).  Operand chunks are gathered through the index maps into shared
 // memory with cp.async, chunk c + 1 while chunk c is multiplied, running along whichever index is
-// contiguous in the operand, so that a warp reads whole sectors.  Both scales are applied to the sums;
-// where they are too large for that (the products of unscaled entries could leave FP32's range) to the
-// gathered entries.
+// contiguous in the operand, so that a warp reads whole sectors.  The scales are applied where no product
+// loses range: to the sums while the unscaled products are the larger ones, else together to B's entries (the
+// products are then those of scaled operands) or, for exponents so large that unscaled entries could leave
+// FP32's range, to the entries of both.  Each thread scales the entries that it copied itself, before the
+// barrier that publishes them.
 // Bound by the FMA pipe (56 % of it at two blocks per SM) and by the last wave of tiles, which run alone
 // on their SMs: 128 x 64 tiles with 8 x 4 outputs a thread spent as much per multiply-add and had the
 // longer tail.  Measured, a 64 x 64 x 512 complex64 tile: 236 k cycles, 308 k with register-staged gathers
@@ -777,6 +779,8 @@ __device__ void tile_gemm(const StepDesc &d, int64_t tile, const JobPtrs &j, cha
     step_scales(d, j, eA, eB);
     constexpr int kLate = sizeof(T) == 4 ? 40 : 120;   // |exponents| up to which the sums are scaled
     const bool late = eA > -kLate && eA < kLate && eB > -kLate && eB < kLate;
+    const int32_t es = eA + eB;
+    const T sA = pow2<T>(-eA), sB = pow2<T>(late ? -es : -eB);   // A: !late; B: !late or es < 0
     const C *__restrict__ A = operand<C>(d, j, true);
     const C *__restrict__ B = operand<C>(d, j, false);
     C *__restrict__ Cp = reinterpret_cast<C *>(j.arena) + d.c_off;
@@ -827,6 +831,21 @@ __device__ void tile_gemm(const StepDesc &d, int64_t tile, const JobPtrs &j, cha
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
+    auto scale_own = [&](int st) {
+        C *a = As + st * stage, *b = a + KC * PA;
+        if (!late) {
+#pragma unroll
+            for (int r = 0; r < RA; ++r) {
+                const int i = tid + r * kThreads, o = a_k ? i % KC * PA + i / KC : i / TM * PA + i % TM;
+                a[o] = cscale(a[o], sA);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            const int i = tid + r * kThreads, o = b_k ? i % KC * PB + i / KC : i / TN * PB + i % TN;
+            b[o] = cscale(b[o], sB);
+        }
+    };
     koffs(0, 0);
     koffs(1, 1);
     __syncthreads();
@@ -843,16 +862,11 @@ __device__ void tile_gemm(const StepDesc &d, int64_t tile, const JobPtrs &j, cha
         const int ahead = slot == 2 ? 0 : slot + 1;
         if (c + 2 < nch) koffs(c + 2, ahead);
         asm volatile("cp.async.wait_group 0;" ::: "memory");
+        if (!late || es < 0) scale_own(c & 1);
         __syncthreads();   // chunk c is there, and chunk c - 1's stage is free
         if (c + 1 < nch) gather((c + 1) & 1, slot);
         slot = ahead;
         C *cur = As + (c & 1) * stage;
-        if (!late) {
-            const T sA = pow2<T>(-eA), sB = pow2<T>(-eB);
-#pragma unroll 1
-            for (int i = tid; i < stage; i += kThreads) cur[i] = cscale(cur[i], i < KC * PA ? sA : sB);
-            __syncthreads();
-        }
         const C *Ak = cur + ks * TK * PA + ty, *Bk = cur + KC * PA + ks * TK * PB + tx;
 #pragma unroll
         for (int kk = 0; kk < TK; ++kk) {
@@ -867,8 +881,8 @@ __device__ void tile_gemm(const StepDesc &d, int64_t tile, const JobPtrs &j, cha
                 for (int jj = 0; jj < RN; ++jj) cfma(acc[i][jj], a[i], b[jj]);
         }
     }
-    if (late) {
-        const T s = pow2<T>(-eA - eB);
+    if (late && es > 0) {
+        const T s = pow2<T>(-es);
 #pragma unroll
         for (int i = 0; i < RM; ++i)
 #pragma unroll

@@ -555,3 +555,42 @@ def test_staged_step_scales_only_its_own_operand(tnsa, shape, magnitude):
     ref, scale = ((x @ y @ b) * d).sum(), ((np.abs(x) @ np.abs(y) @ np.abs(b)) * np.abs(d)).sum()
     # one rounding per leaf and stored step, two per term of the sums over 16 and K, 16 in the dot
     assert abs(m * 2.0 ** e - ref) <= (2 * (K + 16) + 24) * 2.0 ** -24 * scale
+
+
+def _one_output_far_below(precision, exps, shape, depth):
+    """Leaves a (M x K) and b (K x N) with max-abs exponents `exps`, row 1 of a and column 2 of b 2^-depth lower,
+    and a closing tensor that takes the output (1, 2) alone: that output, 2^-(2 depth) of the others, has to keep
+    its own relative accuracy.  Also its value over 2^(exps - 2 depth) and the bound of its error."""
+    M, N, K = shape
+    rng = np.random.default_rng(sum(shape))
+    a, b = (rng.uniform(0.5, 1, s) + 1j * rng.uniform(0.5, 1, s) for s in ((M, K), (K, N)))
+    ref, terms = a[1] @ b[:, 2], np.abs(a[1]) @ np.abs(b[:, 2])
+    a[1] *= 2.0 ** -depth
+    b[:, 2] *= 2.0 ** -depth
+    d = np.zeros((N, M), np.complex128)
+    d[2, 1] = 1.0
+    net = tni.Network([a * 2.0 ** exps[0], b * 2.0 ** exps[1], d], np.array([(0, 1, 1, 0), (1, 1, 2, 0), (2, 1, 0, 0)], np.int32),
+                      np.zeros(3, np.int32), ["t"] * 3)
+    # two roundings per term of the complex sum over K, the leaves, the stored step and 16 in the closing dot
+    return net, [(0, 1), (3, 2)], ref, (2 * K + 24) * (2.0 ** -24 if precision == "c64" else 2.0 ** -53 * 4) * terms
+
+
+def _check_far_below(tnsa, net, steps, ref, bound, precision, exp, budget=0):
+    h = tnsa.tn_build(net)
+    c = tnsa.tn_ctx_create(0)
+    tnsa.tn_ctx_set_config(c, local_budget=budget)
+    m, e, _ = tnsa.tn_contract(c, h, tnsa.tn_plan_import(h, steps), precision)
+    got = complex(math.ldexp(m.real, int(e) - exp), math.ldexp(m.imag, int(e) - exp))
+    assert abs(got - ref) <= bound
+
+
+# register-tiled steps (64 x 64, 128 x 32, 16 x 16 with a long shared index, 32 x 32 complex128): exponents around
+# those up to which the scales are applied to the sums, of one sign and of both
+@pytest.mark.parametrize("shape", [(70, 65, 100), (129, 31, 70), (17, 5, 300)])
+@pytest.mark.parametrize("precision,exps,depth", [
+    ("c64", (0, 0), 33), ("c64", (-39, -38), 33), ("c64", (-20, -20), 50), ("c64", (39, 38), 50), ("c64", (39, -39), 50),
+    ("c64", (-39, 12), 50), ("c64", (-40, -40), 33), ("c64", (-60, -60), 33), ("c128", (-119, -118), 400),
+    ("c128", (100, -119), 400)])
+def test_register_tiled_steps_keep_small_outputs(tnsa, shape, precision, exps, depth):
+    net, steps, ref, bound = _one_output_far_below(precision, exps, shape, depth)
+    _check_far_below(tnsa, net, steps, ref, bound, precision, sum(exps) - 2 * depth)
