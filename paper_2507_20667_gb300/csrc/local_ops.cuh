@@ -211,9 +211,7 @@ __device__ __forceinline__ float small_pass(const uint32_t *ktab, int32_t K, int
 // A small step computed by `parts` warps, of which the calling one is `part`: C = A * B with A, B and
 // C at any address (shared memory, or global memory in warp programs).  S = 2^lg_split lanes share an
 // output and split its shared index; their partial sums are combined with xor shuffles.  The passes of
-// 32 / S outputs are dealt to the parts.  The operand scales 2^-eA and 2^-eB are applied together on
-// the B side when their product is a normal number (products then round exactly as with separate
-// scaling), else separately.
+// 32 / S outputs are dealt to the parts.  eA, eB: the operands' exponents after leave_out_scale.
 // Bound by instruction issue in large batches and by the chain of dependent operations in small ones;
 // a lane therefore works on two outputs at a time where a step has them, and tabulated steps (all but
 // a few) spend three instructions per operand on addresses.  Measured against one output at a time and
@@ -227,10 +225,9 @@ __device__ __forceinline__ float small_core(const LocalStep &s, const cx_t<T> *A
                                             int32_t eA, int32_t eB, int32_t part, int32_t parts) {
     using C = cx_t<T>;
     const int lane = threadIdx.x & 31;
-    const int32_t es = eA + eB;
-    const bool fold = es > -120 && es < 120;
+    const bool fold = scales_fold(eA, eB);
     const T sA = fold ? (T)1 : pow2<T>(-eA);
-    const T sB = fold ? pow2<T>(-es) : pow2<T>(-eB);
+    const T sB = pow2<T>(fold ? -eA - eB : -eB);
     const int32_t N = s.N, K = s.K, O = s.M * s.N, lg = s.lg_split;
     const int32_t sub = lane & ((1 << lg) - 1), per_pass = 32 >> lg;
     float mx = 0.f;
@@ -306,7 +303,9 @@ __device__ __forceinline__ float small_core(const LocalStep &s, const cx_t<T> *A
 template <typename T>
 __device__ __forceinline__ void local_small(const LocalStep &s, const LocalSmem &L, int32_t part, int32_t parts) {
     using C = cx_t<T>;
-    const int32_t eA = scale_exponent(L.smax[s.sa]), eB = scale_exponent(L.smax[s.sb]);
+    int32_t eA = scale_exponent(L.smax[s.sa]);
+    const int32_t eB = scale_exponent(L.smax[s.sb]);
+    leave_out_scale(eA, eB);
     const float mx = small_core<T>(s, reinterpret_cast<const C *>(L.data) + s.a_off,
                                    reinterpret_cast<const C *>(L.data) + s.b_off,
                                    reinterpret_cast<C *>(L.data) + s.c_off, eA, eB, part, parts);
@@ -358,7 +357,9 @@ __device__ void run_warp_prog(int32_t prog, const JobPtrs &j, char *slice) {
         nxt = fetch(si + 2);
         const LocalStep &s = *reinterpret_cast<const LocalStep *>(slice + (si & 1) * sizeof(LocalStep));
         const int2 ma = slot[s.sa], mb = slot[s.sb];
-        const int32_t eA = scale_exponent((uint32_t)ma.x), eB = scale_exponent((uint32_t)mb.x);
+        int32_t eA = scale_exponent((uint32_t)ma.x);
+        const int32_t eB = scale_exponent((uint32_t)mb.x);
+        leave_out_scale(eA, eB);
         const int32_t e = ma.y + eA + mb.y + eB;
         const bool out = s.flags & LFLAG_C_OUT;
         C *Cp = out ? reinterpret_cast<C *>(j.arena) + root_c_off : data + s.c_off;

@@ -109,6 +109,18 @@ template <> __device__ __forceinline__ double pow2<double>(int32_t e) {
     return __longlong_as_double((long long)(e + 1023) << 52);
 }
 
+// Staged and small steps spend no multiplication on A's scale where none is needed: both scales go on B (fold),
+// whose entries only grow by that when A's exponent is negative -- the products are those of scaled operands -- and
+// a positive exponent of A is left out (set to 0: products, sums and stored values are larger by 2^eA, which their
+// max-abs and exponents then say).  Neither costs range: scaling B down by A's exponent would, entries far
+// below B's largest would become subnormal.  Exponents of 60 or more scale each operand on its own.
+__device__ __forceinline__ void leave_out_scale(int32_t &eA, int32_t eB) {
+    if (eA > 0 && eA < 60 && eB > -60 && eB < 60) eA = 0;
+}
+__device__ __forceinline__ bool scales_fold(int32_t eA, int32_t eB) {
+    return eA <= 0 && eA > -60 && eB > -60 && eB < 60;
+}
+
 __device__ __forceinline__ float absmax2(float2 v) { return fmaxf(fabsf(v.x), fabsf(v.y)); }
 __device__ __forceinline__ float absmax2(double2 v) { return (float)fmax(fabs(v.x), fabs(v.y)); }
 
@@ -332,9 +344,9 @@ __device__ __forceinline__ void tile_small(const StepDesc &d, const JobPtrs &j, 
     const int32_t N = (int32_t)d.N, K = (int32_t)d.K, O = (int32_t)d.M * N;
     int32_t eA, eB;
     step_scales(d, j, eA, eB);
-    const int32_t es = eA + eB;
-    const bool fold = es > -120 && es < 120;
-    const float sA = fold ? 1.f : pow2<float>(-eA), sB = fold ? pow2<float>(-es) : pow2<float>(-eB);
+    leave_out_scale(eA, eB);
+    const bool fold = scales_fold(eA, eB);
+    const float sA = fold ? 1.f : pow2<float>(-eA), sB = pow2<float>(fold ? -eA - eB : -eB);
     const float2 *__restrict__ A = operand<float2>(d, j, true);
     const float2 *__restrict__ B = operand<float2>(d, j, false);
     float2 *__restrict__ Cp = reinterpret_cast<float2 *>(j.arena) + d.c_off;
@@ -486,9 +498,8 @@ __device__ float rows_smem_core(const StepHead &d, const JobPtrs &j, char *smem,
     if (tid < K) kat[tid] = __ldg(tab + M + tid);
     int32_t onext[kAheadPer];   // where the next step's B entries are
     if (c_in_smem) b_ahead_offsets(*next, j, onext);
-    // both scales on B where that keeps its entries normal numbers, else A's on A
-    const bool fold = eA > -60 && eA < 60 && eB > -60 && eB < 60;
-    const float sB = fold ? pow2<float>(-eA - eB) : pow2<float>(-eB);
+    const bool fold = scales_fold(eA, eB);
+    const float sB = pow2<float>(fold ? -eA - eB : -eB);
     C *raw = As + kRowsSmemElems;
     if (!a_res) asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (ahead) {   // each thread reads what it copied itself
@@ -611,9 +622,8 @@ __device__ float rows_smem_small(const StepHead &d, const JobPtrs &j, char *dyn,
         b_ahead_offsets(*next, j, onext);
         b_ahead_copy(*next, j, As + kRowsSmemElems, onext);
     }
-    const int32_t es = eA + eB;
-    const bool fold = es > -120 && es < 120;
-    const float sA = fold ? 1.f : pow2<float>(-eA), sB = fold ? pow2<float>(-es) : pow2<float>(-eB);
+    const bool fold = scales_fold(eA, eB);
+    const float sA = fold ? 1.f : pow2<float>(-eA), sB = pow2<float>(fold ? -eA - eB : -eB);
     const uint32_t row = act ? (uint32_t)__ldg(tab + o / N) : 0u, carry = p2 ? 0u : ~0u;
     const C *B = operand<C>(d, j, false) + (act ? __ldg(tab + M + 2 * K + o % N) : 0);
     SmallSum<float> sum;
@@ -656,14 +666,15 @@ __device__ __forceinline__ void tile_rows_smem(const StepDesc &d, const JobPtrs 
                                                float *red) {
     int32_t eA, eB;
     step_scales(d, j, eA, eB);
+    leave_out_scale(eA, eB);
     rows_smem_any<false>(d, j, smem, dyn, red, eA, eB, false, false, nullptr, nullptr);
     if (threadIdx.x == 0) write_exponent(d, j, eA, eB);
 }
 
 // A chain of staged steps linked by chain_next, run by one block of the persistent kernel: the first
 // step reads A from the arena, each later one takes the previous step's C, kept in shared memory,
-// as its A, and the last writes its C to the arena.  The per-step power-of-two scaling is
-// unchanged: a continuation's A exponent comes from the block max of the previous C, which is the
+// as its A, and the last writes its C to the arena.  The per-step power-of-two scaling is that of the
+// separate steps: a continuation's A exponent comes from the block max of the previous C, which is the
 // value the separate steps would publish, so results are bit-identical to running the steps one
 // by one; the exponents of the inner nodes stay in registers and only the last node's max-abs and
 // exponent are written.  The heads of the steps are fetched two steps ahead into a ring of three, and
@@ -706,6 +717,7 @@ __device__ __forceinline__ int32_t rows_chain(const StepDesc &d, const JobPtrs &
             next_max = __ldcg(j.maxbits + next->node_b);
             next_exp = __ldcg(j.exp2 + next->node_b);
         }
+        leave_out_scale(eA, eB);
         const float cmax = rows_smem_any<PROF>(cur, j, smem, dyn, red, eA, eB, n > 0, n > 0, next, prof);
         const int32_t xc = xa + eA + xb + eB;
         if (!next) {

@@ -594,3 +594,29 @@ def _check_far_below(tnsa, net, steps, ref, bound, precision, exp, budget=0):
 def test_register_tiled_steps_keep_small_outputs(tnsa, shape, precision, exps, depth):
     net, steps, ref, bound = _one_output_far_below(precision, exps, shape, depth)
     _check_far_below(tnsa, net, steps, ref, bound, precision, sum(exps) - 2 * depth)
+
+
+# small steps on their own and in programs: exponents of either sign, operands with entries far below the largest
+@pytest.mark.parametrize("shape", [(16, 16, 16), (20, 6, 30), (3, 5, 7)])
+@pytest.mark.parametrize("exps", [(0, 0), (100, 0), (59, -30), (0, 100), (-59, 40), (-80, 19), (70, 50)])
+@pytest.mark.parametrize("budget", [0, -1])
+def test_small_steps_keep_small_outputs(tnsa, shape, exps, budget):
+    net, steps, ref, bound = _one_output_far_below("c64", exps, shape, 40)
+    _check_far_below(tnsa, net, steps, ref, bound, "c64", sum(exps) - 80, budget)
+
+
+# staged steps whose A comes from a long sum (exponent 12), B with a column 2^-125 below its largest entry
+@pytest.mark.parametrize("shape", [(16, 12, 16), (200, 16, 16), (256, 32, 32), (128, 64, 40), (101, 50, 45), (511, 17, 3)])
+def test_staged_steps_keep_small_outputs(tnsa, shape):
+    M, N, K = shape
+    rng = np.random.default_rng(M + N)
+    x, y = np.ones((M, 4096), np.complex128), np.ones((4096, 1)) * rng.integers(4, 8, K) / 8 + 0j   # exact sums
+    b = rng.uniform(0.5, 1, (K, N)) + 0j
+    ref = (x[1] @ y @ b[:, 2]).real
+    b[:, 2] *= 2.0 ** -125
+    d = np.zeros((M, N), np.complex128)
+    d[1, 2] = 1.0
+    net = tni.Network([x, y, b, d], np.array([(0, 1, 1, 0), (1, 1, 2, 0), (0, 0, 3, 0), (2, 1, 3, 1)], np.int32),
+                      np.zeros(4, np.int32), ["t"] * 4)
+    # two roundings per term of the sum over K, the leaves, the stored steps and 16 in the closing dot
+    _check_far_below(tnsa, net, [(0, 1), (4, 2), (5, 3)], ref, (2 * K + 24) * 2.0 ** -24 * ref, "c64", -125)
