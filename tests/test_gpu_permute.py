@@ -86,3 +86,16 @@ def test_permute_tile_edges(env, case, elem):
     got = d_out.cpu().numpy()
     assert np.array_equal(got[shift * elem:(n + shift) * elem], want)
     assert not got[:shift * elem].any() and not got[(n + shift) * elem:].any()
+
+
+# more than 2^31 - 1 elements that cannot be widened: 64-bit offsets in the tiles and in the runs
+@pytest.mark.parametrize("dims,perm", [((46349, 46337), (1, 0)), ((1291, 1301, 1307), (2, 1, 0)), ((1291, 1301, 1307), (1, 0, 2)),
+                                       ((130127, 1273, 13), (1, 0, 2))])
+def test_permute_more_elements_than_32_bits(env, dims, perm):
+    torch, tnsa, ctx = env
+    x = torch.randint(0, 256, dims, dtype=torch.uint8, device="cuda")
+    out = torch.zeros(x.numel(), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    tnsa.tn_permute(ctx, x.data_ptr(), out.data_ptr(), 1, dims, perm)
+    tnsa.tn_ctx_synchronize(ctx)
+    assert torch.equal(out.view([dims[p] for p in perm]), x.permute(*perm))
