@@ -25,11 +25,11 @@ struct PermPlan {
 // One tile: `inner` (or a chunk of it) x group A x group B x group C.  A is a run of the output's
 // innermost axes, B a run of the input's innermost axes outside A, C further axes of the output
 // that fill the tile where A and B cannot (they block each other in a swap of two short axes; they
-// are not needed when the surviving inner run is long).  The last axis of each group may be cut into
-// chunks; the chunk numbers and all other axes form the tile index.  A block reads a tile with
-// consecutive threads along (inner, B) -- contiguous in the input -- and writes it along (inner, A)
-// -- contiguous in the output -- through shared memory, or straight from registers when the two
-// orders agree (no A or no B).
+// are not needed when the surviving inner run is
+// long).  The last axis of each group may be cut into chunks; the chunk numbers and all other axes
+// form the tile index.  A block reads a tile with consecutive threads along (inner, B) -- the input's
+// order -- and writes it along (inner, A) -- the output's order -- through shared memory, or straight
+// from registers when the two orders agree (no A or no B).
 // Bound by HBM.  Everything that depends on the position inside the tile (two offsets and a
 // shared-memory index per element) is computed once per block, which then moves up to kTileRun
 // tiles: only a base changes from tile to tile, the next tile's loads are in flight while the
@@ -38,22 +38,30 @@ struct PermPlan {
 // indices were divided out per element); reversed but for rows of 16 to 512 bytes 164-176 us (470-860
 // us when each row was copied by a group of lanes); (37, 5, 129, 3, 61) complex128 shuffled 29 us
 // (70 us with 32 x 32 tiles of one axis pair, mostly empty).
+struct TileAxis {
+    int64_t in, out;                            // strides
+    uint32_t dim;                               // extent inside the tile, or number of tiles along the axis
+    uint32_t below;                             // tile index: product of the dims before
+};
+// The kernel's parameters.  Every block reads them before its first load, so the axes are packed: with an array of
+// 32 axes for each group (2.3 KB) a block of a small or ragged tensor spent longer on its parameters and tables than
+// on its data ((83910, 88) complex64 transposed 39 us, 34 us packed).
 struct TilePerm {
     int32_t ti, ta, tb, tc;                     // tile edges
     int32_t pitch;                              // shared-memory row of tb * ti elements, odd
     int32_t direct;                             // read and write order agree: no shared memory
     uint32_t mi, ma, mb;                        // ceil(2^32 / edge), 0 for an edge of 1
     int32_t na, nb, nc, nr;                     // axes of each group, innermost first, and of the tile index
-    int32_t adim[kMaxRank], bdim[kMaxRank], cdim[kMaxRank];   // extents inside the tile
-    int64_t ain[kMaxRank], bout[kMaxRank], cin[kMaxRank], cout[kMaxRank];
-    uint32_t rdim[kMaxRank + 4], rbelow[kMaxRank + 4];        // tile index: dims, product of those before
-    int64_t rin[kMaxRank + 4], rout[kMaxRank + 4];
-    int32_t cut[4];                             // tile-index axis that numbers the chunks of inner, A, B, C (-1: whole)
-    int64_t cutdim[4];                          // the cut axis' extent
-    int32_t cutlen[4];                          // and its chunk length
-    int32_t before[4];                          // product of the group's tile extents before the cut axis
     uint32_t n_tiles;
     int32_t run;                                // tiles per block
+    int32_t lanes;                              // lanes that add up a tile's base: nr up to a power of two, at most 32
+    struct Cut {
+        int64_t dim;                            // the cut axis' extent
+        int32_t axis;                           // tile-index axis that numbers the chunks (-1: whole)
+        int32_t len;                            // chunk length
+        int32_t before;                         // product of the group's tile extents before the cut axis
+    } cut[4];                                   // of inner, A, B, C
+    TileAxis ax[kMaxRank + 4];                  // of A, B, C and the tile index, one after the other
 };
 constexpr int kTileRun = 8;    // most tiles per block
 constexpr int kTileEdge = 32;  // elements of the runs on both sides
@@ -61,73 +69,82 @@ constexpr int kTileEdge = 32;  // elements of the runs on both sides
 // Quotient of e < 2^16 by an edge d <= 2^12 from m = ceil(2^32 / d): exact, as e d < 2^32.
 __device__ __forceinline__ uint32_t quot(uint32_t e, uint32_t m) { return m ? __umulhi(e, m) : e; }
 
-__device__ __forceinline__ int64_t digits_off(int32_t idx, int32_t n, const int32_t *dim, const int64_t *str) {
-    int64_t off = 0;
+// Offsets in the input and in the output of a multi-index below the product of n axes' extents.
+__device__ __forceinline__ void digits_off(uint32_t idx, int32_t n, const TileAxis *ax, int64_t &in, int64_t &out) {
+    in = out = 0;
+#pragma unroll 1
     for (int32_t t = 0; t < n; ++t) {
-        const int32_t q = idx / dim[t];
-        off += (int64_t)(idx - q * dim[t]) * str[t];
+        uint32_t q = 0;
+        if (t + 1 < n) q = idx / ax[t].dim;
+        in += (int64_t)(idx - q * ax[t].dim) * ax[t].in;
+        out += (int64_t)(idx - q * ax[t].dim) * ax[t].out;
         idx = q;
     }
-    return off;
 }
 
 // RAGGED: some cut axis has a short last chunk.  O: type of the offsets inside a tile.
 template <typename E, int PER, bool RAGGED, typename O>
-__global__ void __launch_bounds__(256) k_perm_tile(const E *__restrict__ in, E *__restrict__ out,
+__global__ void __launch_bounds__(256, !RAGGED && sizeof(E) == 16 ? 5 : 0) k_perm_tile(const E *__restrict__ in, E *__restrict__ out,
                                                    const __grid_constant__ TilePerm g) {
     extern __shared__ __align__(16) char dyn[];
     __shared__ int64_t s_base[kTileRun][2];
     __shared__ ushort4 s_lim[kTileRun];   // extents of each tile in inner, A, B, C where short of the edges
     __shared__ int32_t s_edge[kTileRun];  // some extent is short
-    int64_t *s_a = reinterpret_cast<int64_t *>(dyn);
-    int64_t *s_b = s_a + g.ta, *s_ci = s_b + g.tb, *s_co = s_ci + g.tc;
+    O *in_a = reinterpret_cast<O *>(dyn), *in_b = in_a + g.ta, *in_c = in_b + g.tb;   // input offsets of the indices
+    O *out_a = in_c + g.tc, *out_b = out_a + g.ta, *out_c = out_b + g.tb;             // output offsets
+    const TileAxis *A = g.ax, *B = A + g.na, *C = B + g.nb, *R = C + g.nc;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t t0 = blockIdx.x * (uint32_t)g.run, nt = min((uint32_t)g.run, g.n_tiles - t0);
-    // tile bases: a warp per tile, a lane per axis of the tile index (at most 36: two rounds)
-    for (uint32_t t = warp; t < nt; t += 8) {
+    // tile bases: a warp per tile, the last warp first (the first ones compute the tables below), a lane per axis of
+    // the tile index (at most 36: two rounds)
+    for (uint32_t t = 7 - warp; t < nt; t += 8) {
         int64_t si = 0, so = 0;
         uint32_t short_axes = 0;
         uint16_t lim[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) lim[q] = 0xffff;
         for (int x = lane; x < g.nr; x += 32) {
-            const uint32_t d = ((t0 + t) / g.rbelow[x]) % g.rdim[x];
-            si += (int64_t)d * g.rin[x];
-            so += (int64_t)d * g.rout[x];
+            const uint32_t d = ((t0 + t) / R[x].below) % R[x].dim;
+            si += (int64_t)d * R[x].in;
+            so += (int64_t)d * R[x].out;
+            if (RAGGED) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (g.cut[q] == x) {
-                    const int64_t left = g.cutdim[q] - (int64_t)d * g.cutlen[q];
-                    if (left < g.cutlen[q]) {
-                        lim[q] = (uint16_t)(left * g.before[q]);
-                        short_axes = 1;
+                for (int q = 0; q < 4; ++q)
+                    if (g.cut[q].axis == x) {
+                        const int64_t left = g.cut[q].dim - (int64_t)d * g.cut[q].len;
+                        if (left < g.cut[q].len) {
+                            lim[q] = (uint16_t)(left * g.cut[q].before);
+                            short_axes = 1;
+                        }
                     }
-                }
+            }
         }
-        for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll 1
+        for (int o = g.lanes >> 1; o > 0; o >>= 1) {
             si += __shfl_xor_sync(0xffffffffu, si, o);
             so += __shfl_xor_sync(0xffffffffu, so, o);
         }
-        const int edge = __any_sync(0xffffffffu, short_axes != 0);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) lim[q] = (uint16_t)__reduce_min_sync(0xffffffffu, (unsigned)lim[q]);
         if (lane == 0) {
             s_base[t][0] = si;
             s_base[t][1] = so;
-            s_lim[t] = make_ushort4(lim[0], lim[1], lim[2], lim[3]);
-            s_edge[t] = edge;
+        }
+        if (RAGGED) {
+            const int edge = __any_sync(0xffffffffu, short_axes != 0);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) lim[q] = (uint16_t)__reduce_min_sync(0xffffffffu, (unsigned)lim[q]);
+            if (lane == 0) {
+                s_lim[t] = make_ushort4(lim[0], lim[1], lim[2], lim[3]);
+                s_edge[t] = edge;
+            }
         }
     }
-    // the input offset of each A index, the output offset of each B index, both of each C index
+    // the input and output offsets of each A, B and C index
     for (int i = tid; i < g.ta + g.tb + g.tc; i += 256) {
-        if (i < g.ta) {
-            s_a[i] = digits_off(i, g.na, g.adim, g.ain);
-        } else if (i < g.ta + g.tb) {
-            s_b[i - g.ta] = digits_off(i - g.ta, g.nb, g.bdim, g.bout);
-        } else {
-            s_ci[i - g.ta - g.tb] = digits_off(i - g.ta - g.tb, g.nc, g.cdim, g.cin);
-            s_co[i - g.ta - g.tb] = digits_off(i - g.ta - g.tb, g.nc, g.cdim, g.cout);
-        }
+        const bool b = i >= g.ta, c = i >= g.ta + g.tb;
+        int64_t oi, oo;
+        digits_off(c ? i - g.ta - g.tb : b ? i - g.ta : i, c ? g.nc : b ? g.nb : g.na, c ? C : b ? B : A, oi, oo);
+        in_a[i] = (O)oi;
+        out_a[i] = (O)oo;
     }
     __syncthreads();
     // per element of this thread: where it is read (order c, a, b, i) and written (order c, b, a, i)
@@ -144,16 +161,15 @@ __global__ void __launch_bounds__(256) k_perm_tile(const E *__restrict__ in, E *
         if (e < n) {
             uint32_t q = quot(e, g.mi), i = e - q * ti, q2 = quot(q, g.mb), b = q - q2 * tb, c = quot(q2, g.ma),
                      a = q2 - c * ta;
-            rd[u] = (O)(s_a[a] + s_ci[c] + b * ti + i);
+            rd[u] = in_a[a] + in_c[c] + (O)(b * ti + i);
             sr[u] = (c * ta + a) * (uint32_t)g.pitch + b * ti + i;
             if (RAGGED) dr[u] = make_uint2(i | a << 16, b | c << 16);
             q2 = quot(q, g.ma), a = q - q2 * ta, c = quot(q2, g.mb), b = q2 - c * tb;
-            wr[u] = (O)(s_b[b] + s_co[c] + a * ti + i);
+            wr[u] = out_b[b] + out_c[c] + (O)(a * ti + i);
             sr[u] |= ((c * ta + a) * (uint32_t)g.pitch + b * ti + i) << 16;
             if (RAGGED) dw[u] = make_uint2(i | a << 16, b | c << 16);
         }
     }
-    __syncthreads();   // the offset tables give way to the tile
     E *tile = reinterpret_cast<E *>(dyn);
     // inside the extents of tile t (all of it unless the tile is at an edge)
     auto inside = [&](uint32_t t, const uint2 &d) {
@@ -169,6 +185,7 @@ __global__ void __launch_bounds__(256) k_perm_tile(const E *__restrict__ in, E *
             if (rd[u] >= 0 && inside(t, dr[u])) v[u] = __ldg(src + rd[u]);
     };
     load(0);
+    __syncthreads();   // the offset tables give way to the tile
     for (uint32_t t = 0; t < nt; ++t) {
         E *dst = out + s_base[t][1];
         if (g.direct) {
@@ -230,12 +247,7 @@ bool tile_perm(const PermPlan &p, int32_t edge, int32_t area, TilePerm &g) {
         take(B, by_in[ib++]);
         return true;
     };
-    for (int q = 0; q < 4; ++q) {
-        g.cut[q] = -1;
-        g.cutdim[q] = 0;
-        g.cutlen[q] = 1;
-        g.before[q] = 1;
-    }
+    for (TilePerm::Cut &c : g.cut) c = {0, -1, 1, 1};
     // cuts the last axis of a group so that its extent is at most lim
     auto cut = [&](Axes &v, int64_t lim, int q) {
         if (v.n == 0) return;
@@ -243,10 +255,7 @@ bool tile_perm(const PermPlan &p, int32_t edge, int32_t area, TilePerm &g) {
         const int64_t before = prod(v) / last.dim, len = chunk(last.dim, std::max<int64_t>(1, lim / before));
         if (len < last.dim) {
             R.push_back({(last.dim + len - 1) / len, last.in * len, last.out * len});
-            g.cutdim[q] = last.dim;
-            g.cutlen[q] = (int32_t)len;
-            g.cut[q] = R.n - 1;   // index into R, renumbered below
-            g.before[q] = (int32_t)before;
+            g.cut[q] = {last.dim, R.n - 1, (int32_t)len, (int32_t)before};   // index into R, renumbered below
             last.dim = len;
         }
     };
@@ -254,9 +263,7 @@ bool tile_perm(const PermPlan &p, int32_t edge, int32_t area, TilePerm &g) {
     if (ti > area) {
         ti = chunk(p.inner, area);
         R.push_back({(p.inner + ti - 1) / ti, ti, ti});
-        g.cutdim[0] = p.inner;
-        g.cutlen[0] = (int32_t)ti;
-        g.cut[0] = 0;
+        g.cut[0] = {p.inner, 0, (int32_t)ti, 1};
     }
     int64_t lim_a = std::max<int64_t>(1, edge / ti), lim_b = std::max<int64_t>(1, area / (ti * lim_a));
     if (ti >= edge) lim_b = 1;   // long surviving runs: whole rows, in the order of the output (C)
@@ -294,13 +301,9 @@ bool tile_perm(const PermPlan &p, int32_t edge, int32_t area, TilePerm &g) {
     g.na = A.n;
     g.nb = B.n;
     g.nc = C.n;
-    for (int32_t i = 0; i < g.na; ++i) { g.adim[i] = (int32_t)A.a[i].dim; g.ain[i] = A.a[i].in; }
-    for (int32_t i = 0; i < g.nb; ++i) { g.bdim[i] = (int32_t)B.a[i].dim; g.bout[i] = B.a[i].out; }
-    for (int32_t i = 0; i < g.nc; ++i) {
-        g.cdim[i] = (int32_t)C.a[i].dim;
-        g.cin[i] = C.a[i].in;
-        g.cout[i] = C.a[i].out;
-    }
+    TileAxis *ax = g.ax;
+    for (const Axes *v : {&A, &B, &C})
+        for (int32_t i = 0; i < v->n; ++i) *ax++ = {v->a[i].in, v->a[i].out, (uint32_t)v->a[i].dim, 0};
     // the tile index: chunk numbers and the other axes, innermost in the output first, so that
     // consecutive tiles write neighbouring runs
     for (int32_t t = 0; t < p.rank; ++t)
@@ -309,29 +312,27 @@ bool tile_perm(const PermPlan &p, int32_t edge, int32_t area, TilePerm &g) {
     for (int32_t i = 0; i < R.n; ++i) ord[i] = i;
     std::sort(ord, ord + R.n, [&](int32_t x, int32_t y) { return R.a[x].out < R.a[y].out; });
     g.nr = R.n;
+    for (g.lanes = 1; g.lanes < std::min(g.nr, 32);) g.lanes *= 2;
     int64_t tiles = 1;
     int32_t cuts[4] = {-1, -1, -1, -1};
     for (int32_t i = 0; i < g.nr; ++i) {
         const Axis &x = R.a[ord[i]];
-        g.rbelow[i] = (uint32_t)tiles;
         if (x.dim > 0x7fffffffLL || tiles > 0x7fffffffLL / x.dim) return false;
+        *ax++ = {x.in, x.out, (uint32_t)x.dim, (uint32_t)tiles};
         tiles *= x.dim;
-        g.rdim[i] = (uint32_t)x.dim;
-        g.rin[i] = x.in;
-        g.rout[i] = x.out;
         for (int q = 0; q < 4; ++q)
-            if (g.cut[q] == ord[i]) cuts[q] = i;
+            if (g.cut[q].axis == ord[i]) cuts[q] = i;
     }
-    for (int q = 0; q < 4; ++q) g.cut[q] = cuts[q];
+    for (int q = 0; q < 4; ++q) g.cut[q].axis = cuts[q];
     g.n_tiles = (uint32_t)tiles;
-    // several tiles per block once every SM has six blocks
-    g.run = (int32_t)std::min<int64_t>(kTileRun, (tiles + 152 * 6 - 1) / (152 * 6));
     return true;
 }
 
+// per_sm: several tiles per block once every SM has that many blocks.
 template <typename E, int PER, bool RAGGED, typename O>
-cudaError_t launch_tiles(const E *in, E *out, const TilePerm &g, cudaStream_t st) {
-    const size_t tables = (size_t)(g.ta + g.tb + 2 * g.tc) * 8;
+cudaError_t launch_tiles(const E *in, E *out, TilePerm &g, int32_t per_sm, cudaStream_t st) {
+    g.run = (int32_t)std::min<int64_t>(kTileRun, ((int64_t)g.n_tiles + 152 * per_sm - 1) / (152 * per_sm));
+    const size_t tables = (size_t)(g.ta + g.tb + g.tc) * 2 * sizeof(O);
     const size_t smem = std::max(tables, g.direct ? 0 : (size_t)g.tc * g.ta * g.pitch * sizeof(E));
     const unsigned blocks = (g.n_tiles + g.run - 1) / g.run;
     k_perm_tile<E, PER, RAGGED, O><<<blocks, 256, smem, st>>>(in, out, g);
@@ -339,28 +340,30 @@ cudaError_t launch_tiles(const E *in, E *out, const TilePerm &g, cudaStream_t st
 }
 
 // Tiles of 2048 elements of up to 8 bytes where no chunk is short, of 1024 otherwise: a 16-byte element
-// fills 16 KB with 1024, and the bookkeeping of ragged tiles costs registers per element.
+// fills 16 KB with 1024, and the bookkeeping of ragged tiles costs registers per element (four of their blocks of
+// up to 8 bytes an element fit an SM: a target of six left a second wave half empty).
 template <typename E>
 cudaError_t perm_launch(const void *src, void *dst, const PermPlan &p, cudaStream_t st) {
     if (p.total == 0) return cudaSuccess;
     const E *in = static_cast<const E *>(src);
     E *out = static_cast<E *>(dst);
     constexpr int AREA = sizeof(E) <= 8 ? 2048 : 1024;
+    const bool wide = p.total > 0x7fffffffLL;
     TilePerm g;
-    auto ragged = [&]() {
-        bool r = false;
-        for (int q = 0; q < 4; ++q) r = r || (g.cut[q] >= 0 && g.cutdim[q] % g.cutlen[q] != 0);
+    auto whole = [](const TilePerm &t) {
+        bool r = true;
+        for (const TilePerm::Cut &c : t.cut) r = r && (c.axis < 0 || c.dim % c.len == 0);
         return r;
     };
-    const bool wide = p.total > 0x7fffffffLL;
     if (!wide && p.total > 152 * 6 * 1024) {   // enough tiles to choose their size
         if (!tile_perm(p, kTileEdge, AREA, g)) return cudaErrorInvalidValue;
-        if (!ragged()) return launch_tiles<E, AREA / 256, false, int32_t>(in, out, g, st);
+        if (whole(g)) return launch_tiles<E, AREA / 256, false, int32_t>(in, out, g, 6, st);
     }
     if (!tile_perm(p, kTileEdge, 1024, g)) return cudaErrorInvalidValue;
-    if (wide) return launch_tiles<E, 4, true, int64_t>(in, out, g, st);
-    return ragged() ? launch_tiles<E, 4, true, int32_t>(in, out, g, st)
-                    : launch_tiles<E, 4, false, int32_t>(in, out, g, st);
+    if (!wide && whole(g)) return launch_tiles<E, 4, false, int32_t>(in, out, g, 6, st);
+    constexpr int32_t per_sm = sizeof(E) == 16 ? 6 : 4;
+    return wide ? launch_tiles<E, 4, true, int64_t>(in, out, g, per_sm, st)
+                : launch_tiles<E, 4, true, int32_t>(in, out, g, per_sm, st);
 }
 
 // The fused plan of a permutation; false if it has too many axes.
