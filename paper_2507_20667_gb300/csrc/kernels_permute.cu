@@ -23,9 +23,9 @@ struct PermPlan {
 };
 
 // One tile: `inner` (or a chunk of it) x group A x group B x group C.  A is a run of the output's
-// innermost axes, B a run of the input's innermost axes outside A, C further axes of the output
-// that fill the tile where A and B cannot (they block each other in a swap of two short axes; they
-// are not needed when the surviving inner run is
+// innermost axes, B a run of the input's innermost axes, each without the axes that the other one has
+// taken (these are whole inside the tile, so the run goes on past them), C further axes of the output
+// that fill the tile where A and B cannot (they are not needed when the surviving inner run is
 // long).  The last axis of each group may be cut into chunks; the chunk numbers and all other axes
 // form the tile index.  A block reads a tile with consecutive threads along (inner, B) -- the input's
 // order -- and writes it along (inner, A) -- the output's order -- through shared memory, or straight
@@ -37,7 +37,9 @@ struct PermPlan {
 // 2^26 complex64: all axes reversed 169 us, 6.4 TB/s (297 us with 64 x 64 tiles, one per block, whose
 // indices were divided out per element); reversed but for rows of 16 to 512 bytes 164-176 us (470-860
 // us when each row was copied by a group of lanes); (37, 5, 129, 3, 61) complex128 shuffled 29 us
-// (70 us with 32 x 32 tiles of one axis pair, mostly empty).
+// (70 us with 32 x 32 tiles of one axis pair, mostly empty).  Shuffles that put one of the input's
+// last axes first in the output need the runs that go on past the other group's axes: one of 2^26
+// complex64 takes 168 us, 249 us with runs that stop there (64 bytes and less).
 struct TileAxis {
     int64_t in, out;                            // strides
     uint32_t dim;                               // extent inside the tile, or number of tiles along the axis
@@ -161,11 +163,11 @@ __global__ void __launch_bounds__(256, !RAGGED && sizeof(E) == 16 ? 5 : 0) k_per
         if (e < n) {
             uint32_t q = quot(e, g.mi), i = e - q * ti, q2 = quot(q, g.mb), b = q - q2 * tb, c = quot(q2, g.ma),
                      a = q2 - c * ta;
-            rd[u] = in_a[a] + in_c[c] + (O)(b * ti + i);
+            rd[u] = in_a[a] + in_b[b] + in_c[c] + (O)i;
             sr[u] = (c * ta + a) * (uint32_t)g.pitch + b * ti + i;
             if (RAGGED) dr[u] = make_uint2(i | a << 16, b | c << 16);
             q2 = quot(q, g.ma), a = q - q2 * ta, c = quot(q2, g.mb), b = q2 - c * tb;
-            wr[u] = out_b[b] + out_c[c] + (O)(a * ti + i);
+            wr[u] = out_a[a] + out_b[b] + out_c[c] + (O)i;
             sr[u] |= ((c * ta + a) * (uint32_t)g.pitch + b * ti + i) << 16;
             if (RAGGED) dw[u] = make_uint2(i | a << 16, b | c << 16);
         }
@@ -237,12 +239,16 @@ bool tile_perm(const PermPlan &p, int32_t edge, int32_t area, TilePerm &g) {
         v.push_back({p.odim[t], p.istride[t], p.ostride[t]});
         used[t] = 1;
     };
-    auto grow_a = [&](int64_t lim) {
+    // a run goes on past the axes of the other group unless that one's last axis is about to be cut (past a cut
+    // axis nothing is contiguous)
+    auto grow_a = [&](int64_t lim, int64_t lim_b) {
+        while (ia >= 0 && used[ia] && prod(B) <= lim_b) --ia;
         if (ia < 0 || used[ia] || prod(A) >= lim) return false;
         take(A, ia--);
         return true;
     };
-    auto grow_b = [&](int64_t lim) {
+    auto grow_b = [&](int64_t lim, int64_t lim_a) {
+        while (ib < p.rank && used[by_in[ib]] && prod(A) <= lim_a) ++ib;
         if (ib >= p.rank || used[by_in[ib]] || prod(B) >= lim) return false;
         take(B, by_in[ib++]);
         return true;
@@ -268,17 +274,17 @@ bool tile_perm(const PermPlan &p, int32_t edge, int32_t area, TilePerm &g) {
     int64_t lim_a = std::max<int64_t>(1, edge / ti), lim_b = std::max<int64_t>(1, area / (ti * lim_a));
     if (ti >= edge) lim_b = 1;   // long surviving runs: whole rows, in the order of the output (C)
     for (bool more = true; more;) {   // in turn, so that neither takes all the short axes
-        const bool ga = grow_a(lim_a), gb = grow_b(lim_b);
+        const bool ga = grow_a(lim_a, lim_b), gb = grow_b(lim_b, lim_a);
         more = ga || gb;
     }
     // a group that is blocked short of its edge leaves more of the tile to the other
     if (ti < edge && prod(A) < lim_a) {
         lim_b = std::max(lim_b, area / (ti * prod(A)));
-        while (grow_b(lim_b)) {}
+        while (grow_b(lim_b, lim_a)) {}
     }
     if (ti < edge && prod(B) < lim_b) {
         lim_a = std::max(lim_a, area / (ti * prod(B)));
-        while (grow_a(lim_a)) {}
+        while (grow_a(lim_a, lim_b)) {}
     }
     cut(A, lim_a, 1);
     cut(B, lim_b, 2);

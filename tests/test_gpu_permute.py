@@ -88,6 +88,29 @@ def test_permute_tile_edges(env, case, elem):
     assert not got[:shift * elem].any() and not got[(n + shift) * elem:].any()
 
 
+# paths chosen by size: tiles whose input axes lie partly in the output's group, whole or about to be cut
+PATH_CASES = [
+    ((2,) * 14, (4, 7, 0, 9, 13, 3, 11, 1, 8, 5, 2, 6, 10, 12)), ((3, 2, 5, 7, 2, 3), (4, 2, 0, 3, 5, 1)), ((37, 33, 3, 20, 5), (0, 2, 3, 4, 1)),
+]
+
+
+@pytest.mark.parametrize("case", range(len(PATH_CASES)))
+@pytest.mark.parametrize("elem", [1, 2, 4, 8, 16])
+def test_permute_paths_by_size(env, case, elem):
+    torch, tnsa, ctx = env
+    dims, perm = PATH_CASES[case]
+    n = int(np.prod(dims))
+    src = np.random.default_rng(case).integers(0, 256, n * elem, dtype=np.uint8)
+    d_in = torch.from_numpy(src).cuda()
+    d_out = torch.zeros((n + 2) * elem, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    tnsa.tn_permute(ctx, d_in.data_ptr(), d_out.data_ptr() + elem * (elem < 16), elem, dims, perm)
+    tnsa.tn_ctx_synchronize(ctx)
+    got = d_out.cpu().numpy()[elem * (elem < 16):]
+    want = src.reshape(*dims, elem).transpose(*perm, len(dims)).reshape(-1)
+    assert np.array_equal(got[:n * elem], want) and not got[n * elem:].any()
+
+
 # more than 2^31 - 1 elements that cannot be widened: 64-bit offsets in the tiles and in the runs
 @pytest.mark.parametrize("dims,perm", [((46349, 46337), (1, 0)), ((1291, 1301, 1307), (2, 1, 0)), ((1291, 1301, 1307), (1, 0, 2)),
                                        ((130127, 1273, 13), (1, 0, 2))])
