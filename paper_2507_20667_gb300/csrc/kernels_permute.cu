@@ -1,7 +1,8 @@
 // Axis permutation of a row-major tensor (the "T" of TTGT, Section 5.1): out axis t = in axis
 // perm[t].  Moves bytes only, so it is exact for any payload.  Axes that stay adjacent and in
 // order are fused first, and a surviving innermost axis widens the element (up to 16 bytes) where
-// the buffers are aligned for it.  One kernel then moves tiles: see TilePerm.
+// the buffers are aligned for it.  One kernel then moves tiles (see TilePerm), one copies long surviving runs
+// that fill no tile (k_perm_runs).
 #include <algorithm>
 #include <cstdint>
 
@@ -209,6 +210,73 @@ __global__ void __launch_bounds__(256, !RAGGED && sizeof(E) == 16 ? 5 : 0) k_per
     }
 }
 
+// Long surviving runs of which no whole number fills a tile: G lanes copy one run (or a chunk of it), kRunLoads loads
+// in flight each, sharing the division of its number into axes; with fewer lanes for short runs a warp has
+// several runs in flight.  Bound by HBM from 4 bytes an element, by the loads issued below that.  Ragged tiles of
+// 1024 elements (or tiles half empty) kept too few bytes in flight: (1291, 1301, 1307) with its outer axes exchanged
+// 5.4 ms in complex64 (6.5 TB/s) and 1.3 ms in bytes, 14.1 and 7.4 ms in tiles, 5.5 and 2.1 ms with a warp
+// per run and four loads; (1436, 1437, 65) complex64 358 us, 771 and 810 us.
+constexpr int kRunChunk = 2048, kRunLoads = 6;
+template <typename E, int G>
+__global__ void __launch_bounds__(256) k_perm_runs(const E *__restrict__ in, E *__restrict__ out,
+                                                   const __grid_constant__ TilePerm g) {
+    constexpr uint32_t per = 32 / G;
+    constexpr int U = kRunLoads;
+    const uint32_t lane = threadIdx.x & 31, sub = lane & (G - 1), grp = lane / G;
+    const uint32_t warps = gridDim.x * 8;
+    for (uint32_t t0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * per; t0 < g.n_tiles; t0 += warps * per) {
+        const uint32_t t = t0 + grp;
+        int64_t si = 0, so = 0;
+        for (int x = sub; x < g.nr; x += G) {
+            const uint32_t d = (t / g.ax[x].below) % g.ax[x].dim;
+            si += (int64_t)d * g.ax[x].in;
+            so += (int64_t)d * g.ax[x].out;
+        }
+#pragma unroll 1
+        for (int o = g.lanes >> 1; o > 0; o >>= 1) {
+            si += __shfl_xor_sync(0xffffffffu, si, o);
+            so += __shfl_xor_sync(0xffffffffu, so, o);
+        }
+        const E *src = in + __shfl_sync(0xffffffffu, si, lane - sub);
+        E *dst = out + __shfl_sync(0xffffffffu, so, lane - sub);
+        int32_t n = t < g.n_tiles ? g.ti : 0;
+        if (g.cut[0].axis >= 0)   // the chunk number is the first axis
+            n = (int32_t)min((int64_t)n, g.cut[0].dim - (int64_t)(t % g.ax[0].dim) * n);
+        for (int32_t i0 = sub; i0 < n; i0 += G * U) {
+            E v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (i0 + G * u < n) v[u] = __ldg(src + i0 + G * u);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (i0 + G * u < n) dst[i0 + G * u] = v[u];
+        }
+    }
+}
+
+// The tile index of plan p's runs; false where they are too few to fill the GPU (2048 are six warps an SM in each
+// pass; 812 runs of 20011 complex64 numbers took the same time either way).
+bool run_perm(const PermPlan &p, TilePerm &g) {
+    const int64_t chunks = (p.inner + kRunChunk - 1) / kRunChunk;
+    g.ti = (int32_t)((p.inner + chunks - 1) / chunks);
+    g.cut[0] = {p.inner, chunks > 1 ? 0 : -1, g.ti, 1};
+    int64_t tiles = 1;
+    g.nr = 0;
+    auto axis = [&](int64_t dim, int64_t in, int64_t out) {
+        if (dim > 0x7fffffffLL || tiles > 0x7fffffffLL / dim) return false;
+        g.ax[g.nr++] = {in, out, (uint32_t)dim, (uint32_t)tiles};
+        tiles *= dim;
+        return true;
+    };
+    if (chunks > 1 && !axis(chunks, g.ti, g.ti)) return false;
+    for (int32_t t = p.rank - 1; t >= 0; --t)
+        if (!axis(p.odim[t], p.istride[t], p.ostride[t])) return false;
+    for (g.ta = 8; g.ta < 32 && g.ta * kRunLoads < g.ti;) g.ta *= 2;
+    for (g.lanes = 1; g.lanes < std::min(g.nr, g.ta);) g.lanes *= 2;
+    g.n_tiles = (uint32_t)tiles;
+    return tiles >= 2048;
+}
+
 // Builds the tiles of plan p: runs of about `edge` elements on both sides, at most `area` elements.
 // false if the tensor has too many of them.
 bool tile_perm(const PermPlan &p, int32_t edge, int32_t area, TilePerm &g) {
@@ -345,6 +413,14 @@ cudaError_t launch_tiles(const E *in, E *out, TilePerm &g, int32_t per_sm, cudaS
     return cudaGetLastError();
 }
 
+template <typename E, int G>
+cudaError_t launch_runs(const E *in, E *out, const TilePerm &g, cudaStream_t st) {
+    constexpr unsigned per = 8 * (32 / G);
+    const unsigned nb = std::min<unsigned>((g.n_tiles + per - 1) / per, 152 * 8);
+    k_perm_runs<E, G><<<nb, 256, 0, st>>>(in, out, g);
+    return cudaGetLastError();
+}
+
 // Tiles of 2048 elements of up to 8 bytes where no chunk is short, of 1024 otherwise: a 16-byte element
 // fills 16 KB with 1024, and the bookkeeping of ragged tiles costs registers per element (four of their blocks of
 // up to 8 bytes an element fit an SM: a target of six left a second wave half empty).
@@ -354,19 +430,27 @@ cudaError_t perm_launch(const void *src, void *dst, const PermPlan &p, cudaStrea
     const E *in = static_cast<const E *>(src);
     E *out = static_cast<E *>(dst);
     constexpr int AREA = sizeof(E) <= 8 ? 2048 : 1024;
-    const bool wide = p.total > 0x7fffffffLL;
+    const bool wide = p.total > 0x7fffffffLL, runs = p.inner >= kTileEdge;
     TilePerm g;
-    auto whole = [](const TilePerm &t) {
-        bool r = true;
+    // no chunk is short, and of long surviving runs of up to 8 bytes an element enough fit in to fill the tile
+    auto whole = [runs](const TilePerm &t, int32_t area) {
+        bool r = !runs || sizeof(E) == 16 || 4 * t.ti * t.tc >= 3 * area;
         for (const TilePerm::Cut &c : t.cut) r = r && (c.axis < 0 || c.dim % c.len == 0);
         return r;
     };
     if (!wide && p.total > 152 * 6 * 1024) {   // enough tiles to choose their size
         if (!tile_perm(p, kTileEdge, AREA, g)) return cudaErrorInvalidValue;
-        if (whole(g)) return launch_tiles<E, AREA / 256, false, int32_t>(in, out, g, 6, st);
+        if (whole(g, AREA)) return launch_tiles<E, AREA / 256, false, int32_t>(in, out, g, 6, st);
     }
     if (!tile_perm(p, kTileEdge, 1024, g)) return cudaErrorInvalidValue;
-    if (!wide && whole(g)) return launch_tiles<E, 4, false, int32_t>(in, out, g, 6, st);
+    if (!wide && whole(g, 1024)) return launch_tiles<E, 4, false, int32_t>(in, out, g, 6, st);
+    if (TilePerm r; runs && run_perm(p, r)) {
+        switch (r.ta) {
+            case 8: return launch_runs<E, 8>(in, out, r, st);
+            case 16: return launch_runs<E, 16>(in, out, r, st);
+            default: return launch_runs<E, 32>(in, out, r, st);
+        }
+    }
     constexpr int32_t per_sm = sizeof(E) == 16 ? 6 : 4;
     return wide ? launch_tiles<E, 4, true, int64_t>(in, out, g, per_sm, st)
                 : launch_tiles<E, 4, true, int32_t>(in, out, g, per_sm, st);

@@ -88,9 +88,12 @@ def test_permute_tile_edges(env, case, elem):
     assert not got[:shift * elem].any() and not got[(n + shift) * elem:].any()
 
 
-# paths chosen by size: tiles whose input axes lie partly in the output's group, whole or about to be cut
+# paths chosen by size: tiles whose input axes lie partly in the output's group, whole or about to be cut; long
+# surviving runs copied run by run (8, 16 and 32 lanes a run, runs cut into chunks, one run too few)
 PATH_CASES = [
     ((2,) * 14, (4, 7, 0, 9, 13, 3, 11, 1, 8, 5, 2, 6, 10, 12)), ((3, 2, 5, 7, 2, 3), (4, 2, 0, 3, 5, 1)), ((37, 33, 3, 20, 5), (0, 2, 3, 4, 1)),
+    ((45, 46, 33), (1, 0, 2)), ((64, 33, 65), (1, 0, 2)), ((13, 17, 11, 131), (2, 0, 1, 3)), ((33, 32, 2049), (1, 0, 2)),
+    ((23, 89, 33), (1, 0, 2)),
 ]
 
 
