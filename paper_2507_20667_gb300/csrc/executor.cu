@@ -2369,10 +2369,10 @@ tn_status tn_permute(tn_ctx *ctx, const void *d_in, void *d_out, int32_t elem_by
     if (rank < 0 || rank > 32) return fail(TN_EINVAL, "rank must be in [0, 32]");
     if (elem_bytes != 1 && elem_bytes != 2 && elem_bytes != 4 && elem_bytes != 8 && elem_bytes != 16)
         return fail(TN_EINVAL, "elem_bytes must be 1, 2, 4, 8 or 16");
-    std::vector<int> seen(rank, 0);
+    uint32_t seen = 0;
     for (int32_t t = 0; t < rank; ++t) {
-        if (perm[t] < 0 || perm[t] >= rank || seen[perm[t]]) return fail(TN_EINVAL, "perm is not a permutation");
-        seen[perm[t]] = 1;
+        if (perm[t] < 0 || perm[t] >= rank || (seen >> perm[t] & 1u)) return fail(TN_EINVAL, "perm is not a permutation");
+        seen |= 1u << perm[t];
         if (dims[t] < 1) return fail(TN_EINVAL, "dims must be >= 1");
     }
     CK(cudaSetDevice(ctx->device));

@@ -93,6 +93,7 @@ def test_permute_tile_edges(env, case, elem):
 # transpositions of two long axes (with and without other axes, large ones of 16 bytes alone)
 PATH_CASES = [
     ((2,) * 14, (4, 7, 0, 9, 13, 3, 11, 1, 8, 5, 2, 6, 10, 12)), ((3, 2, 5, 7, 2, 3), (4, 2, 0, 3, 5, 1)), ((37, 33, 3, 20, 5), (0, 2, 3, 4, 1)),
+    ((2, 1) * 16, tuple(range(31, -1, -1))),
     ((45, 46, 33), (1, 0, 2)), ((64, 33, 65), (1, 0, 2)), ((13, 17, 11, 131), (2, 0, 1, 3)), ((33, 32, 2049), (1, 0, 2)),
     ((23, 89, 33), (1, 0, 2)),
     ((97, 65), (1, 0)), ((129, 3, 63), (2, 1, 0)), ((64, 127), (1, 0)), ((32, 31, 95), (2, 0, 1)), ((1500, 1401), (1, 0)),
