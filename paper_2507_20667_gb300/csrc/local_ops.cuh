@@ -211,7 +211,7 @@ __device__ __forceinline__ float small_pass(const uint32_t *ktab, int32_t K, int
 // A small step computed by `parts` warps, of which the calling one is `part`: C = A * B with A, B and
 // C at any address (shared memory, or global memory in warp programs).  S = 2^lg_split lanes share an
 // output and split its shared index; their partial sums are combined with xor shuffles.  The passes of
-// 32 / S outputs are dealt to the parts.  eA, eB: the operands' exponents after leave_out_scale.
+// 32 / S outputs are dealt to the parts.  eA, eB, fold: the operands' exponents after leave_out_scale, its result.
 // Bound by instruction issue in large batches and by the chain of dependent operations in small ones;
 // a lane therefore works on two outputs at a time where a step has them, and tabulated steps (all but
 // a few) spend three instructions per operand on addresses.  Measured against one output at a time and
@@ -222,12 +222,10 @@ __device__ __forceinline__ float small_pass(const uint32_t *ktab, int32_t K, int
 // Returns the warp-wide max-abs of its part of C (every lane).
 template <typename T>
 __device__ __forceinline__ float small_core(const LocalStep &s, const cx_t<T> *A, const cx_t<T> *B, cx_t<T> *Cp,
-                                            int32_t eA, int32_t eB, int32_t part, int32_t parts) {
+                                            int32_t eA, int32_t eB, bool fold, int32_t part, int32_t parts) {
     using C = cx_t<T>;
     const int lane = threadIdx.x & 31;
-    const bool fold = scales_fold(eA, eB);
-    const T sA = fold ? (T)1 : pow2<T>(-eA);
-    const T sB = pow2<T>(fold ? -eA - eB : -eB);
+    const T sA = pow2_scale<T>(-eA), sB = pow2_scale<T>(fold ? -eA - eB : -eB);   // sA where the scales do not fold
     const int32_t N = s.N, K = s.K, O = s.M * s.N, lg = s.lg_split;
     const int32_t sub = lane & ((1 << lg) - 1), per_pass = 32 >> lg;
     float mx = 0.f;
@@ -305,10 +303,10 @@ __device__ __forceinline__ void local_small(const LocalStep &s, const LocalSmem 
     using C = cx_t<T>;
     int32_t eA = scale_exponent(L.smax[s.sa]);
     const int32_t eB = scale_exponent(L.smax[s.sb]);
-    leave_out_scale(eA, eB);
+    const bool fold = leave_out_scale(eA, eB);
     const float mx = small_core<T>(s, reinterpret_cast<const C *>(L.data) + s.a_off,
                                    reinterpret_cast<const C *>(L.data) + s.b_off,
-                                   reinterpret_cast<C *>(L.data) + s.c_off, eA, eB, part, parts);
+                                   reinterpret_cast<C *>(L.data) + s.c_off, eA, eB, fold, part, parts);
     if ((threadIdx.x & 31) == 0) {
         if (parts > 1) atomicMax(L.smax + s.sc, __float_as_uint(mx));
         else L.smax[s.sc] = __float_as_uint(mx);
@@ -359,11 +357,11 @@ __device__ void run_warp_prog(int32_t prog, const JobPtrs &j, char *slice) {
         const int2 ma = slot[s.sa], mb = slot[s.sb];
         int32_t eA = scale_exponent((uint32_t)ma.x);
         const int32_t eB = scale_exponent((uint32_t)mb.x);
-        leave_out_scale(eA, eB);
+        const bool fold = leave_out_scale(eA, eB);
         const int32_t e = ma.y + eA + mb.y + eB;
         const bool out = s.flags & LFLAG_C_OUT;
         C *Cp = out ? reinterpret_cast<C *>(j.arena) + root_c_off : data + s.c_off;
-        const float mx = small_core<T>(s, data + s.a_off, data + s.b_off, Cp, eA, eB, 0, 1);
+        const float mx = small_core<T>(s, data + s.a_off, data + s.b_off, Cp, eA, eB, fold, 0, 1);
         if (lane == 0) {
             if (out) {
                 j.maxbits[root_node] = __float_as_uint(mx);

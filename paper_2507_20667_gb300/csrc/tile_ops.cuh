@@ -109,16 +109,26 @@ template <> __device__ __forceinline__ double pow2<double>(int32_t e) {
     return __longlong_as_double((long long)(e + 1023) << 52);
 }
 
+// The same without the limits, for scales: scale_exponent is in [-126, 126], and sums of two are taken only where
+// each is below 60 in magnitude.
+template <typename T> __device__ __forceinline__ T pow2_scale(int32_t e);
+template <> __device__ __forceinline__ float pow2_scale<float>(int32_t e) { return __int_as_float((e + 127) << 23); }
+template <> __device__ __forceinline__ double pow2_scale<double>(int32_t e) {
+    return __longlong_as_double((long long)(e + 1023) << 52);
+}
+
 // Staged and small steps spend no multiplication on A's scale where none is needed: both scales go on B (fold),
 // whose entries only grow by that when A's exponent is negative -- the products are those of scaled operands -- and
 // a positive exponent of A is left out (set to 0: products, sums and stored values are larger by 2^eA, which their
 // max-abs and exponents then say).  Neither costs range: scaling B down by A's exponent would, entries far
-// below B's largest would become subnormal.  Exponents of 60 or more scale each operand on its own.
-__device__ __forceinline__ void leave_out_scale(int32_t &eA, int32_t eB) {
-    if (eA > 0 && eA < 60 && eB > -60 && eB < 60) eA = 0;
-}
+// below B's largest would become subnormal.  Exponents of 60 or more scale each operand on its own (false).
 __device__ __forceinline__ bool scales_fold(int32_t eA, int32_t eB) {
-    return eA <= 0 && eA > -60 && eB > -60 && eB < 60;
+    return (uint32_t)(eA + 59) < 119u && (uint32_t)(eB + 59) < 119u;
+}
+__device__ __forceinline__ bool leave_out_scale(int32_t &eA, int32_t eB) {
+    const bool fold = scales_fold(eA, eB);
+    if (fold) eA = min(eA, 0);
+    return fold;
 }
 
 __device__ __forceinline__ float absmax2(float2 v) { return fmaxf(fabsf(v.x), fabsf(v.y)); }
@@ -344,8 +354,7 @@ __device__ __forceinline__ void tile_small(const StepDesc &d, const JobPtrs &j, 
     const int32_t N = (int32_t)d.N, K = (int32_t)d.K, O = (int32_t)d.M * N;
     int32_t eA, eB;
     step_scales(d, j, eA, eB);
-    leave_out_scale(eA, eB);
-    const bool fold = scales_fold(eA, eB);
+    const bool fold = leave_out_scale(eA, eB);
     const float sA = fold ? 1.f : pow2<float>(-eA), sB = pow2<float>(fold ? -eA - eB : -eB);
     const float2 *__restrict__ A = operand<float2>(d, j, true);
     const float2 *__restrict__ B = operand<float2>(d, j, false);
