@@ -142,10 +142,10 @@ def kernel_sources_sha():
 
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of the three contraction kernels of one
-# run of the headline workload (k_warp 195.8 MB + k_local 321.9 MB + k_persist 3736.1 MB per
+# run of the headline workload (k_warp 196.0 MB + k_local 321.4 MB + k_persist 1007.2 MB per
 # launch, mean of two runs), from one ncu capture of `bench.py` at the default batch
 # (profiles/traffic_brickwork24_batch2432.md); valid for the kernel sources with this hash.
-TRAFFIC = {"sources_sha": "41dac86b20f80667", "batch": 2432, "bytes_per_run": 4253917056}
+TRAFFIC = {"sources_sha": "1e857e42f81f8b44", "batch": 2432, "bytes_per_run": 1524680576}
 
 
 def measured_peaks():
