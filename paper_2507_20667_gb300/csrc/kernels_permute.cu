@@ -278,11 +278,10 @@ bool run_perm(const PermPlan &p, TilePerm &g) {
 }
 
 // The transposition of two long axes (the output's innermost and the input's innermost), one 32 x 32 tile of
-// them a block: no tables, next to no set-up.  Taken where the general kernel's tiles would be ragged, at least three
-// quarters of the 32 x 32 ones are full, and the elements are of 16 bytes or at most 2^21: small tensors are bound by
-// a block's set-up ((1354, 625) complex64 hot in L2 4.2 us, 10.3 us in ragged tiles; (1158, 1430) complex128 8.3
-// and 12.4 us); from 4 M elements of up to 8 bytes the general kernel's longer runs win ((6887, 5204) float32 89
-// and 111 us).
+// them a block: no tables, next to no set-up, eight blocks an SM.  Taken where the general kernel's tiles would be ragged
+// and the 32 x 32 ones are at least half full.  Against the ragged tiles it takes 0.5 to 0.9 of the time over 300 shapes
+// of 2^18 to 2^27 elements (at a fill of 0.52 to 0.56 as much or less): (1354, 625) complex64 hot in L2 4.2 us, 10.3 us;
+// (745, 12738) float32 18.5 us, 28 us; (6466, 2337) complex64 39 us, 56 us; (1158, 1430) complex128 12.4 us, 16.4 us.
 template <typename E>
 __global__ void __launch_bounds__(256) k_perm_plane(const E *__restrict__ in, E *__restrict__ out,
                                                     const __grid_constant__ TilePerm g) {
@@ -317,14 +316,14 @@ __global__ void __launch_bounds__(256) k_perm_plane(const E *__restrict__ in, E 
 }
 
 // The two axes of plan p and its other ones, where k_perm_plane takes them (see there).
-bool plane_perm(const PermPlan &p, int32_t elem, TilePerm &g) {
-    if (p.inner != 1 || p.rank < 2 || (elem < 16 && p.total > (2 << 20))) return false;
+bool plane_perm(const PermPlan &p, TilePerm &g) {
+    if (p.inner != 1 || p.rank < 2) return false;
     const int32_t a = p.rank - 1;
     int32_t b = 0;
     while (p.istride[b] != 1) ++b;
     const int64_t da = p.odim[a], db = p.odim[b], ta = (da + 31) / 32, tb = (db + 31) / 32;
     int64_t tiles = p.total / (da * db);
-    if (da > 0x7fffffffLL || db > 0x7fffffffLL || 4 * da * db < 3 * (ta * 32) * (tb * 32)) return false;
+    if (da > 0x7fffffffLL || db > 0x7fffffffLL || 2 * da * db < (ta * 32) * (tb * 32)) return false;
     if (ta > 0x7fffffffLL / tb || tiles > 0x7fffffffLL / (ta * tb)) return false;
     tiles *= ta * tb;
     g.ta = (int32_t)ta;
@@ -513,7 +512,7 @@ cudaError_t perm_launch(const void *src, void *dst, const PermPlan &p, cudaStrea
             default: return launch_runs<E, 32>(in, out, r, st);
         }
     }
-    if (TilePerm r; plane_perm(p, sizeof(E), r)) {
+    if (TilePerm r; plane_perm(p, r)) {
         k_perm_plane<E><<<r.n_tiles, 256, 0, st>>>(in, out, r);
         return cudaGetLastError();
     }

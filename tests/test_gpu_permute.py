@@ -90,13 +90,14 @@ def test_permute_tile_edges(env, case, elem):
 
 # paths chosen by size: tiles whose input axes lie partly in the output's group, whole or about to be cut; long
 # surviving runs copied run by run (8, 16 and 32 lanes a run, runs cut into chunks, one run too few);
-# transpositions of two long axes (with and without other axes, large ones of 16 bytes alone)
+# transpositions of two long axes (with and without other axes, tiles just over and under half full)
 PATH_CASES = [
     ((2,) * 14, (4, 7, 0, 9, 13, 3, 11, 1, 8, 5, 2, 6, 10, 12)), ((3, 2, 5, 7, 2, 3), (4, 2, 0, 3, 5, 1)), ((37, 33, 3, 20, 5), (0, 2, 3, 4, 1)),
     ((2, 1) * 16, tuple(range(31, -1, -1))),
     ((45, 46, 33), (1, 0, 2)), ((64, 33, 65), (1, 0, 2)), ((13, 17, 11, 131), (2, 0, 1, 3)), ((33, 32, 2049), (1, 0, 2)),
     ((23, 89, 33), (1, 0, 2)),
     ((97, 65), (1, 0)), ((129, 3, 63), (2, 1, 0)), ((64, 127), (1, 0)), ((32, 31, 95), (2, 0, 1)), ((1500, 1401), (1, 0)),
+    ((33, 700), (1, 0)), ((33, 33), (1, 0)), ((17, 5, 64), (2, 1, 0)),
 ]
 
 
