@@ -58,6 +58,7 @@ struct CompileOpts {
     int32_t tc_min_m = 64, tc_min_n = 32, tc_min_k = 16;
     int32_t tc_tile_n = 0;            // dense-step tile width: 0 automatic (64 if N <= 64), 64, 128
     bool rows_chains = true;
+    int32_t jobs = 1;                 // contractions of the batch (sizes tiles; no value depends on it)
 };
 
 // Compile (network structure, plan): the global dataflow step list, the subtree programs and the

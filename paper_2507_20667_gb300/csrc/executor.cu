@@ -286,10 +286,15 @@ size_t plan_memory(const Plan &plan, int32_t n, const std::vector<size_t> &bytes
 // Rows per work tile of a global ROWS step: large enough to amortise the tile's fixed cost
 // (descriptor, scales, B staging, completion fence), 16 rows per thread at most.  Complex128 tiles hold
 // about 8192 multiply-adds instead: at the FP64 rate these take 16 k cycles, twice the fixed cost, and a
-// 4096 x 16 x 4 step in one tile held up its job for 140 k cycles while other SMs idled.
-int32_t rows_per_tile(int64_t M, int64_t N, int64_t K, int32_t elem) {
+// 4096 x 16 x 4 step in one tile held up its job for 140 k cycles while other SMs idled (one job 352 us, 61 us in
+// tiles of 256 rows).  Where the batch has rows for four larger tiles per SM they are taken: the fixed cost of
+// small ones is 10 to 16 % of a full batch (1024 jobs of 4096 x 4 x 16: 2.98 ms, 2.51 ms).  A row's value does not
+// depend on its tile.
+int32_t rows_per_tile(int64_t M, int64_t N, int64_t K, int32_t elem, int64_t jobs) {
     int64_t rows = 4096;
-    if (elem == 16) rows = std::min(rows, std::max<int64_t>(kThreads, 8192 / (N * K) / kThreads * kThreads));
+    if (elem == 16)
+        rows = std::min(rows, std::max({(int64_t)kThreads, 8192 / (N * K) / kThreads * kThreads,
+                                        jobs * M / (4 * 152) / kThreads * kThreads}));
     return (int32_t)std::max<int64_t>(1, std::min(M, rows));
 }
 
@@ -937,7 +942,7 @@ tn_status tn::compile(Compiled &c, const Net &net, const Plan &plan, const Compi
             c.counts[STEP_ROWS]++;
         } else if (N <= kRowsMaxN && K <= kRowsMaxK && K * N <= kRowsMaxKN) {
             d.kind = STEP_ROWS;
-            d.tile_rows = rows_per_tile(M, N, K, elem);
+            d.tile_rows = rows_per_tile(M, N, K, elem, opt.jobs);
             d.ntiles = (int32_t)((M + d.tile_rows - 1) / d.tile_rows);
             c.steps.push_back(d);
             c.counts[STEP_ROWS]++;
@@ -1483,6 +1488,7 @@ tn_status batch_create(tn_ctx *ctx, int32_t n, const tn_net *const *nets, const 
     b->job_comp.assign(n, -1);
     // compile every distinct (structure, plan) once
     CompileOpts copt = compile_opts(ctx->cfg, prec, b->c128);
+    copt.jobs = n;
     std::unordered_map<std::string, int32_t> seen;
     for (int32_t i = 0; i < n; ++i) {
         const Net &net = nets[i]->impl;

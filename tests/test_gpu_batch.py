@@ -276,3 +276,32 @@ def test_large_leaves_at_any_alignment(sizes):
     assert (st == 0).all()
     # leaves, products, bursts of 16 products and the stored dots are rounded to 24 bits
     assert (np.abs(m * np.exp2(e) - refs) <= 2 * 24 * 2.0 ** -24 * np.array(scales)).all()
+
+
+@pytest.mark.parametrize("shape", [(4096, 4, 16), (3000, 5, 7)])
+def test_complex128_rows_are_the_same_in_any_batch(shape):
+    """The rows of a complex128 step are cut into tiles by the size of the batch (256 to 4096 rows); a row's value
+    does not depend on its tile: the same bits alone and among 200 jobs, which equal numpy's."""
+    from paper_2507_20667_gb300 import tnsa
+    M, N, K = shape
+    rng = np.random.default_rng(M)
+
+    def normal(*s):
+        return rng.standard_normal(s) + 1j * rng.standard_normal(s)
+    a, b, c = normal(M, K), normal(K, N), normal(N, M)
+    net = tni.Network([a, b, c], np.array([(0, 1, 1, 0), (1, 1, 2, 0), (2, 1, 0, 0)], np.int32), np.zeros(3, np.int32), ["t"] * 3)
+    h = tnsa.tn_build(net)
+    plan = tnsa.tn_plan_import(h, [(0, 1), (3, 2)])
+    out = []
+    for jobs in (1, 40, 200):
+        ctx = tnsa.tn_ctx_create(0)
+        tnsa.tn_ctx_set_config(ctx, local_budget=0)
+        batch = tnsa.tn_batch_create(ctx, [h] * jobs, [plan] * jobs, "c128")
+        tnsa.tn_batch_run(batch)
+        m, e, st = tnsa.tn_batch_results(batch)
+        assert (st == 0).all() and (m == m[0]).all() and (e == e[0]).all()
+        out.append((m[0], int(e[0])))
+    assert out[0] == out[1] == out[2]
+    ref, scale = np.einsum("ij,ji->", a @ b, c), np.einsum("ij,ji->", np.abs(a) @ np.abs(b), np.abs(c))
+    # sums of K products, then of M N / 2048 bursts of eight per thread
+    assert abs(out[0][0] * 2.0 ** out[0][1] - ref) <= (2 * K + 64 + M * N / 2048) * 2.0 ** -52 * scale
