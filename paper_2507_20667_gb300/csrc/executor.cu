@@ -964,11 +964,13 @@ tn_status tn::compile(Compiled &c, const Net &net, const Plan &plan, const Compi
             c.counts[STEP_TC]++;
         } else {
             d.kind = STEP_TILE;
-            // complex64: few outputs and a long shared index split the latter over thread groups, narrow
+            // complex64: few outputs and a long shared index split the latter over thread groups, in 32 x 32
+            // tiles where 16 x 16 ones would be eight and more (see tile_gemm), narrow
             // outputs (N <= 32) leave no thread to compute padding; complex128, bound by FP64 (a tile's
             // 32 x 32 x 16 takes 33 k cycles), uses small tiles so that a small batch fills the SMs
             d.tile_rows = elem != 8                        ? TILE_C128
-                          : M * N <= 4096 && K >= 256      ? TILE_LONG_K
+                          : M * N <= 4096 && K >= 256
+                              ? (N > 16 && M > 16 && (M + 15) / 16 * ((N + 15) / 16) >= 8 ? TILE_LONG_K32 : TILE_LONG_K)
                           : N <= tile_n(TILE_NARROW)       ? TILE_NARROW
                                                            : TILE_SQUARE;
             const int64_t tm = tile_m(d.tile_rows), tn = tile_n(d.tile_rows);

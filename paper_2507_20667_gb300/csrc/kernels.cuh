@@ -253,7 +253,7 @@ cudaError_t launch_permute(const void *src, void *dst, int32_t elem_bytes, int32
 // Tiling constants shared by the compiler and the kernels.
 constexpr int kThreads = 256;
 // CUDA-core GEMM tiles (StepDesc.tile_rows of a TILE step): output rows and columns.
-enum TileShape : int32_t { TILE_SQUARE = 0, TILE_NARROW = 1, TILE_LONG_K = 2, TILE_C128 = 3 };
+enum TileShape : int32_t { TILE_SQUARE = 0, TILE_NARROW = 1, TILE_LONG_K = 2, TILE_C128 = 3, TILE_LONG_K32 = 4 };
 constexpr int tile_m(int shape) { return shape == TILE_SQUARE ? 64 : shape == TILE_NARROW ? 128 : shape == TILE_LONG_K ? 16 : 32; }
 constexpr int tile_n(int shape) { return shape == TILE_SQUARE ? 64 : shape == TILE_LONG_K ? 16 : 32; }
 constexpr int kRowsMaxKN = 1024, kRowsMaxK = 64, kRowsMaxN = 16;

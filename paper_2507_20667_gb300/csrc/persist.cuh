@@ -7,7 +7,7 @@
 // progresses (co-residency of the grid is not needed).  A block claims its next tile while the
 // current one runs.  A chain of ROWS steps that fit shared memory is one work item, its tensor kept there
 // between the steps.  In complex64 the kernel takes all 128 registers that two blocks per SM leave a thread
-// and spills 136 bytes (ptxas -v).  Each storage type is instantiated in its own translation unit
+// and spills 148 bytes (ptxas -v).  Each storage type is instantiated in its own translation unit
 // (kernels_persist_f32.cu, kernels_persist_f64.cu).
 #pragma once
 

@@ -777,7 +777,9 @@ __device__ __forceinline__ void tile_rows_dispatch(const StepDesc &d, int64_t ti
 // on their SMs: 128 x 64 tiles with 8 x 4 outputs a thread spent as much per multiply-add and had the
 // longer tail.  Measured, a 64 x 64 x 512 complex64 tile: 236 k cycles, 308 k with register-staged gathers
 // along the rows.  Few outputs with a long shared index take KS = 4: 8 x 8 x 512 took 250 k cycles in a
-// 64 x 64 tile and takes 45 k.
+// 64 x 64 tile and takes 45 k in 16 x 16.  From eight such tiles on their threads, two rows and two columns each, wait
+// for shared memory too long in a full batch: 64 x 64 x 512 takes 32 x 32 tiles of 4 x 4 outputs a thread, one contraction
+// 51 us (37 us in 16 x 16, 96 us in 64 x 64), 1024 of them 0.64 ms (1.05 and 0.50 ms).
 template <typename T, int TM, int TN, int RM, int RN, int TK, int KS>
 __device__ void tile_gemm(const StepDesc &d, int64_t tile, const JobPtrs &j, char *smem, float *red) {
     using C = cx_t<T>;
@@ -949,6 +951,12 @@ __device__ void tile_gemm(const StepDesc &d, int64_t tile, const JobPtrs &j, cha
     }
     publish_max(mx, j.maxbits + d.node_c, red);
     if (tile == 0 && threadIdx.x == 0) write_exponent(d, j, eA, eB);
+}
+
+// Out of line: rare, and inlined it moved the other tile shapes about (1 % of a dense complex64 step).
+static __device__ __noinline__ void tile_long32(const StepDesc &d, int64_t tile, const JobPtrs &j, char *smem,
+                                                float *red) {
+    tile_gemm<float, 32, 32, 4, 4, 4, 4>(d, tile, j, smem, red);
 }
 
 // ------------------------------------------------------------------------------ DOT
@@ -1179,6 +1187,7 @@ __device__ __forceinline__ void run_tile(const StepDesc &d, int64_t tile, const 
             if constexpr (sizeof(T) == 4) {
                 if (d.tile_rows == TILE_NARROW) tile_gemm<T, 128, 32, 4, 4, 8, 1>(d, tile, j, smem, red);
                 else if (d.tile_rows == TILE_LONG_K) tile_gemm<T, 16, 16, 2, 2, 8, 4>(d, tile, j, smem, red);
+                else if (d.tile_rows == TILE_LONG_K32) tile_long32(d, tile, j, smem, red);
                 else tile_gemm<T, 64, 64, 4, 4, 8, 1>(d, tile, j, smem, red);
             } else {
                 tile_gemm<T, 32, 32, 2, 2, 8, 1>(d, tile, j, smem, red);

@@ -620,3 +620,28 @@ def test_staged_steps_keep_small_outputs(tnsa, shape):
                       np.zeros(4, np.int32), ["t"] * 4)
     # two roundings per term of the sum over K, the leaves, the stored steps and 16 in the closing dot
     _check_far_below(tnsa, net, [(0, 1), (4, 2), (5, 3)], ref, (2 * K + 24) * 2.0 ** -24 * ref, "c64", -125)
+
+
+# few outputs with a long shared index, more of them than eight 16 x 16 tiles: 32 x 32 tiles, the index split four ways
+@pytest.mark.parametrize("shape", [(64, 64, 256), (33, 33, 257), (128, 32, 300), (63, 65, 1001), (49, 48, 512), (17, 240, 260)])
+@pytest.mark.parametrize("transposed", [(0, 0), (1, 0), (0, 1)])
+@pytest.mark.parametrize("magnitude", [1.0, 2.0 ** 60, 2.0 ** -30])
+def test_long_shared_index_in_wider_tiles(tnsa, shape, transposed, magnitude):
+    M, N, K = shape
+    rng = np.random.default_rng(M + N + K)
+
+    def normal(*s):
+        return (rng.standard_normal(s) + 1j * rng.standard_normal(s)) / math.sqrt(2)
+    a, b, c = normal(M, K) * magnitude, normal(K, N), normal(N, M)
+    ta, tb = transposed
+    edges = [(0, 0 if ta else 1, 1, 1 if tb else 0), (1, 0 if tb else 1, 2, 0), (2, 1, 0, 1 if ta else 0)]
+    net = tni.Network([a.T.copy() if ta else a, b.T.copy() if tb else b, c], np.array(edges, np.int32),
+                      np.zeros(3, np.int32), ["t"] * 3)
+    h = tnsa.tn_build(net)
+    ctx = tnsa.tn_ctx_create(0)
+    tnsa.tn_ctx_set_config(ctx, local_budget=0)
+    m, e, _ = tnsa.tn_contract(ctx, h, tnsa.tn_plan_import(h, [(0, 1), (3, 2)]), "c64")
+    ref = np.einsum("ij,ji->", a @ b, c)
+    scale = np.einsum("ij,ji->", np.abs(a) @ np.abs(b), np.abs(c))
+    # two roundings per term of the complex sum over K, the leaves, the stored step and 16 in the closing dot
+    assert abs(m * 2.0 ** e - ref) <= (2 * K + 24) * 2.0 ** -24 * scale
