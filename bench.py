@@ -142,10 +142,10 @@ def kernel_sources_sha():
 
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of the three contraction kernels of one
-# run of the headline workload (k_warp 195.7 MB + k_local 321.7 MB + k_persist 1007.4 MB per
+# run of the headline workload (k_warp 195.6 MB + k_local 321.5 MB + k_persist 1008.1 MB per
 # launch, mean of two runs), from one ncu capture of `bench.py` at the default batch
 # (profiles/traffic_brickwork24_batch2432.md); valid for the kernel sources with this hash.
-TRAFFIC = {"sources_sha": "4658974f0d559e4c", "batch": 2432, "bytes_per_run": 1524780160}
+TRAFFIC = {"sources_sha": "fb54f64625bec9e2", "batch": 2432, "bytes_per_run": 1525326720}
 
 
 def measured_peaks():
